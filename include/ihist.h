@@ -70,7 +70,13 @@ enum { IHIST_BIN_MAJOR = 0, IHIST_PIXEL_MAJOR = 1, IHIST_QUAD_MAJOR = 2 };
 typedef struct ihist_plan_s *ihist_plan_t;
 
 /* Tile shape of the fused scan kernel.  Zero fields take the library's
- * default for the frame shape.
+ * default for the frame shape.  A plan that leaves every tiling field zero
+ * (rows_per_band, bins_per_cta, chunks_per_warp, groups_per_cta, ctas_per_sm,
+ * warps_per_cta) may take the two-launch path instead (a count kernel, then
+ * an emit kernel; bin- and quad-major frames up to 12 and 40 megapixels),
+ * which has no tiling of its own: ihist_plan_get_tune then reports the tiling
+ * of the fused kernel for the shape, and passing it back selects that kernel.
+ * Results are the same words either way.
  *   rows_per_band   R, rows one CTA owns (1..255)
  *   bins_per_cta    G, bins one CTA owns (4, 8 or 16; default 4, or for
  *                   pixel-major output 16 (8 with fewer than 16 bins or

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "ihist.h"
+#include "ihist_bands_host.h"
 #include "ihist_host.h"
 #include "ihist_joint.cuh"
 #include "ihist_kernels.h"
@@ -57,6 +58,8 @@ struct ihist_plan_s {
   unsigned int timeout_us;
   int fault_skip_band;
   int overlap;          // launch with programmatic dependent launch
+  bool banded;          // frames go through the two-launch path (ihist_bands.cuh)
+  BandDesc band;        // its shape and workspace
   size_t smem_bytes;
   void *ws;
   size_t ws_bytes;
@@ -241,6 +244,13 @@ static int plan_create(int h, int w, int nbins, int layout, const ihist_tune_t *
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return IHIST_ERR_CUDA;
   const int nchunks = (w + kChunk - 1) / kChunk;
+  // The two-launch path takes plans with no tiling of their own; a tiling
+  // (and the test hook, which lives in its carries) asks for the look-back
+  // kernel.
+  const bool tiled = t.rows_per_band || t.bins_per_cta || t.chunks_per_warp || t.ctas_per_sm || t.groups_per_cta ||
+                     t.warps_per_cta || t.fault_skip_band >= 1;
+  BandDesc band;
+  bool banded = !tiled && bands_shape(h, w, nbins, layout, sms, &band);
   // Pixel-major output: a pixel's counts of one bin group are G contiguous
   // words and the groups of a pixel belong to different CTAs, so larger
   // groups give longer contiguous pieces per pixel record; rows are staged
@@ -376,8 +386,29 @@ static int plan_create(int h, int w, int nbins, int layout, const ihist_tune_t *
   }
   p->ctas_per_sm = t.ctas_per_sm > 0 ? std::min(t.ctas_per_sm, occ) : occ;
 
-  // workspace: control block, flags, column-count aggregates, left counts, inclusive rows
-  const size_t nci = (size_t)p->nbands * p->ngroups * p->nchunks;
+  const int mode = table ? kBinTable : joint ? kBinJoint : kBinUniform;
+  if (banded && table && nbins > 252)  // no byte left for "no bin"
+    for (int v = 0; v < 256; ++v) banded = banded && bin_map[v] >= 0;
+  if (banded) {
+    int optin_b = 0;
+    if (cudaDeviceGetAttribute(&optin_b, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+      delete p;
+      return IHIST_ERR_CUDA;
+    }
+    const int brc = bands_prepare(band, mode, (size_t)optin_b);
+    if (brc == IHIST_ERR_UNSUPPORTED) {
+      banded = false;
+    } else if (brc != IHIST_OK) {
+      delete p;
+      return brc;
+    }
+  }
+  p->banded = banded;
+
+  // workspace: control blocks, then the two-launch path's counts or the
+  // look-back kernel's flags, column-count aggregates, left counts and
+  // inclusive rows
+  const size_t nci = banded ? 0 : (size_t)p->nbands * p->ngroups * p->nchunks;
   size_t off = 0;
   const size_t o_ctrl = off;
   off = align_up(off + sizeof(Ctrl), 256);
@@ -385,7 +416,7 @@ static int plan_create(int h, int w, int nbins, int layout, const ihist_tune_t *
   off = align_up(off + sizeof(Ctrl), 256);
   const size_t o_flags = off;
   off = align_up(off + nci * sizeof(uint32_t), 256);
-  const size_t nhs = nsegs > 1 ? (size_t)p->nbands * p->ngroups * nsegs : 0;  // segment records
+  const size_t nhs = !banded && nsegs > 1 ? (size_t)p->nbands * p->ngroups * nsegs : 0;  // segment records
   const size_t o_hflags = off;
   off = align_up(off + nhs * sizeof(uint32_t), 256);
   const size_t o_cnt = off;
@@ -400,7 +431,9 @@ static int plan_create(int h, int w, int nbins, int layout, const ihist_tune_t *
   if (table) off = align_up(off + 256 * sizeof(uint32_t), 256);
   const size_t o_idx = off;
   p->idx_pitch = align_up((size_t)w, 16);
-  if (joint) off = align_up(off + (size_t)h * p->idx_pitch, 256);
+  if (joint && !banded) off = align_up(off + (size_t)h * p->idx_pitch, 256);
+  const size_t o_band = off;
+  if (banded) off += bands_layout(&band, nullptr);
   p->ws_bytes = off;
   if (cudaMalloc(&p->ws, p->ws_bytes) != cudaSuccess) {
     cudaGetLastError();
@@ -419,7 +452,21 @@ static int plan_create(int h, int w, int nbins, int layout, const ihist_tune_t *
     p->hagg = reinterpret_cast<uint32_t *>(base + o_hagg);
   }
   if (table) p->lut = reinterpret_cast<uint32_t *>(base + o_lut);
-  if (joint) p->idx = reinterpret_cast<uint8_t *>(base + o_idx);
+  if (joint && !banded) p->idx = reinterpret_cast<uint8_t *>(base + o_idx);
+  if (banded) {
+    bands_layout(&band, base + o_band);
+    band.lut = p->lut;
+    band.ctrl = p->ctrl;
+    band.qmul = nbins;
+    if (joint) {
+      band.jc = joint->C;
+      for (int c = 0; c < 4; ++c) {
+        band.jmul[c] = joint->mul[c];
+        band.jstride[c] = joint->stride[c];
+      }
+    }
+    p->band = band;
+  }
   uint32_t host_lut[256];
   for (int v = 0; v < 256; ++v)
     host_lut[v] = table && bin_map[v] >= 0 ? 8u * (uint32_t)bin_map[v] : kNoBin;
@@ -596,7 +643,8 @@ static const CUtensorMap *input_map(ihist_plan_s *p, const uint8_t *d_in, size_t
   return e.ok ? &e.map : nullptr;
 }
 
-// One frame (ihist_compute).  Every scan is launched with programmatic
+// One frame (ihist_compute), through the two-launch path or the look-back
+// kernel.  Every scan is launched with programmatic
 // stream serialization, so its CTAs may start while the previous kernel on
 // the stream finishes; they take their first work item and then wait for
 // that kernel (griddepcontrol.wait) before reading the frame, or, with
@@ -610,6 +658,16 @@ static int compute_frame(ihist_plan_s *p, const uint8_t *d_in, size_t in_pitch, 
   if (((uintptr_t)d_out & 3u) != 0) return IHIST_ERR_INVALID_ARG;
   int rc = check_device(p);
   if (rc != IHIST_OK) return rc;
+  if (p->banded) {
+    BandDesc b = p->band;
+    b.in = d_in;
+    b.pitch = (long long)in_pitch;
+    b.out = d_out;
+    // joint plans never read ahead: their frames may come from the kernel just before
+    b.early = overlap && p->binning != kJoint ? 1 : 0;
+    return launch_bands(b, p->binning == kTable ? kBinTable : p->binning == kJoint ? kBinJoint : kBinUniform, p->layout,
+                        stream);
+  }
   if (p->binning == kJoint) {
     // joint bins first, one byte per pixel; the scan then reads that plane
     int rc2 = launch_joint_index(d_in, (long long)in_pitch, p->H, p->W, p->joint.C, p->joint.mul, p->idx,

@@ -1,0 +1,565 @@
+// ihist_bands.cuh -- the integral histogram of one frame in two launches
+// that wait on nothing inside themselves: band_count_kernel reads the frame
+// once and leaves the counts that every band starts from, band_emit_kernel
+// writes H (Eq. 1 of arXiv 1711.01919).
+//
+// What it is for: the look-back kernel (ihist_scan.cuh) carries counts from
+// band to band through flags in global memory, and a frame that fills only a
+// wave or two of CTAs spends as long on that chain (ticket, count, publish,
+// look back, publish again) as on its stores.  Counting needs no chain: the
+// number of pixels of a bin above a band, in one column, is a sum of the
+// column's counts in the bands above, and those depend on the frame alone.
+// Measured per frame, back to back, look-back kernel -> these two (uniform
+// pixels, GB300): 320x240 x 16 16.9 -> 6.2 us, 640x480 x 32 21.4 -> 11.4,
+// 1280x720 x 32 36 -> 26, 1920x1080 x 64 104.9 -> 85.5 (a plain fill of the
+// same bytes takes 78.5), 1921x1081 x 64 160 -> 92, 3840x2160 x 64 355 -> 329;
+// quad-major 1920x1080 x 64 108 -> 90, 1921x1081 x 64 582 -> 116.
+//
+// Superband: 4 bands of R rows (R = 8, 16 or 32).  A group is 4 bins, packed
+// as the bytes of one word; a chunk is 128 columns.  The count kernel leaves
+//   q    [H][chunks * 128]           each pixel's bin, one byte
+//   pb   [band][group][column]       counts of the column in the bands above
+//                                    this one within its superband (bytes)
+//   sb   [superband][group][column]  counts of the column in the superband
+//   rl   [chunk][group][row]         counts of the row inside the chunk
+//   ct   [band][group][chunk]        counts of the band inside the chunk
+//                                    (16-bit lanes; only when a band is split
+//                                    into width segments)
+// and a band's first row of H follows from pb, the sb above and a scan along
+// the columns.
+#pragma once
+
+#include "ihist_device.cuh"
+
+namespace ihist {
+
+constexpr int kSuper = 4;            // bands per superband
+constexpr int kCountThreads = 512;
+constexpr int kHalf = kChunk / 2;    // columns of a column tile
+constexpr int kColPitch = kHalf + 4;  // bytes between rows of a column tile
+constexpr int kRowPitch = kChunk + 4;  // of a row tile: rows one bank apart, so a warp reads down a column of words without conflicts
+constexpr int kSegWarps = 8;         // chunks of one emit CTA at most
+
+struct BandDesc {
+  const uint8_t *in;
+  long long pitch;
+  uint32_t *out;
+  const uint32_t *lut;  // table plans: 8 * bin of each intensity, or the no-bin mark
+  int jc, jmul[4], jstride[4];  // joint plans: channels, their bins and digit weights (see ihist_joint.cuh)
+  int H, W, B, qmul;
+  int early;            // 1: the frame may be read before the previous grid has completed
+  int R, nbands, nsb, nq, nchunks, nsegs, cps;
+  int split;  // a count thread counts R >> split pixels
+  uint8_t *q;
+  uint32_t *pb, *sb, *rl;
+  uint2 *ct;
+  Ctrl *ctrl;  // checked builds: where a failed store check is latched
+};
+
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// One more in a byte counter of this thread's own (shared memory address).
+__device__ __forceinline__ void bump_byte(uint32_t a) {
+  asm volatile(
+      "{\n\t.reg .u32 n;\n\t"
+      "ld.shared.u8 n, [%0];\n\t"
+      "add.u32 n, n, 1;\n\t"
+      "st.shared.u8 [%0], n;\n\t}" ::"r"(a)
+      : "memory");
+}
+
+enum { kBinUniform = 0, kBinTable = 1, kBinJoint = 2 };
+
+// Bins of four pixels, one byte each.
+template <int MODE>
+__device__ __forceinline__ uint32_t bins4(const BandDesc &f, const uint8_t *s_lut, uint32_t v) {
+  if constexpr (MODE == kBinTable) {
+    return (uint32_t)s_lut[v & 0xffu] | (uint32_t)s_lut[(v >> 8) & 0xffu] << 8 |
+           (uint32_t)s_lut[(v >> 16) & 0xffu] << 16 | (uint32_t)s_lut[v >> 24] << 24;
+  } else {
+    // floor(v * B / 256): two products in 16-bit lanes, v * B <= 255 * 256
+    const uint32_t e = (v & 0x00ff00ffu) * (uint32_t)f.qmul, o = ((v >> 8) & 0x00ff00ffu) * (uint32_t)f.qmul;
+    return ((e >> 8) & 0x00ff00ffu) | (o & 0xff00ff00u);
+  }
+}
+
+// Put the bins of rows r, r + step, .. < nrows (of the rows from y0 on) at
+// columns x .. x+3 into a tile column (and, with to_q, into the plane of
+// bins).  Columns past the frame get bin 0: they lie right of every column
+// that is stored, so no result depends on them.
+template <int MODE>
+__device__ __forceinline__ void load_tile(const BandDesc &f, const uint8_t *s_lut, int y0, int r, int step, int nrows,
+                                          int x, uint32_t *tp, int tstep, bool to_q) {
+  const size_t wpad = (size_t)f.nchunks * kChunk;
+  const uint8_t *src = f.in + (long long)(y0 + r) * f.pitch;
+  uint8_t *qp = f.q + (size_t)(y0 + r) * wpad + x;
+  const long long sstep = (long long)step * f.pitch;
+  const size_t qstep = (size_t)step * wpad;
+  const bool words = MODE != kBinJoint && x + 3 < f.W &&
+                     ((reinterpret_cast<uintptr_t>(f.in) | (uintptr_t)f.pitch) & 3u) == 0;
+  if (words) {
+    src += x;
+#pragma unroll 8
+    for (; r < nrows; r += step) {
+      const uint32_t q = bins4<MODE>(f, s_lut, __ldcg(reinterpret_cast<const unsigned int *>(src)));
+      *tp = q;
+      if (to_q) *reinterpret_cast<uint32_t *>(qp) = q;
+      src += sstep;
+      tp += tstep;
+      qp += qstep;
+    }
+  } else {
+#pragma unroll 2
+    for (; r < nrows; r += step) {
+      uint32_t q = 0u;
+      if constexpr (MODE == kBinJoint) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (x + i < f.W) {
+            uint32_t k = 0u;
+            for (int c = 0; c < f.jc; ++c)
+              k += (((uint32_t)__ldg(src + (x + i) * f.jc + c) * (uint32_t)f.jmul[c]) >> 8) * (uint32_t)f.jstride[c];
+            q |= k << (8 * i);
+          }
+        }
+      } else {
+        uint32_t v = 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (x + i < f.W) v |= (uint32_t)__ldg(src + x + i) << (8 * i);
+        q = bins4<MODE>(f, s_lut, v);
+      }
+      *tp = q;
+      if (to_q) *reinterpret_cast<uint32_t *>(qp) = q;
+      src += sstep;
+      tp += tstep;
+      qp += qstep;
+    }
+  }
+}
+
+// Shared memory of the count kernel: the tile's bins, then one byte counter
+// per bin and thread, as words of 4 bins [nq + 1][512] (thread t's word of
+// group g in bank t mod 32 whatever the pixel, so no access conflicts; the
+// extra word takes values that are in no bin).  A column tile is 64 columns
+// x 8 pieces of R >> split rows, a row tile 128 columns x as many rows as
+// make 512 pieces of R >> split pixels.
+__host__ __device__ inline int col_tile_rows(const BandDesc &f) { return 8 * (f.R >> f.split); }
+__host__ __device__ inline int row_tile_rows(const BandDesc &f) { return 4 * (f.R >> f.split); }
+__host__ __device__ inline size_t count_tile_bytes(const BandDesc &f) {
+  const int col = col_tile_rows(f) * kColPitch, row = row_tile_rows(f) * kRowPitch;
+  return (size_t)(col > row ? col : row);
+}
+__host__ __device__ inline size_t count_smem_bytes(const BandDesc &f) {
+  return count_tile_bytes(f) + (size_t)(f.nq + 1) * kCountThreads * 4;
+}
+
+// Each thread counts R >> split pixels of one column, or of one row, in its
+// own byte counters, so a pixel costs two counter updates in all whatever
+// the number of bins; the CTA then adds its threads' counters up into the
+// columns' and rows' counts.  Grid: x over half chunks, y over column tiles
+// of rows; z = 0 column tiles, 1 row tiles (two per column tile).
+template <int MODE>
+__global__ void __launch_bounds__(kCountThreads, 4) band_count_kernel(const __grid_constant__ BandDesc f) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  __shared__ uint8_t s_lut[MODE == kBinTable ? 256 : 1];
+  if (!f.early) griddep_wait();
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  uint32_t *tile32 = reinterpret_cast<uint32_t *>(smem_raw);
+  uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + count_tile_bytes(f));
+  const size_t wpad = (size_t)f.nchunks * kChunk;
+  const int per = f.R >> f.split;  // pixels one thread counts
+  if constexpr (MODE == kBinTable) {
+    const uint32_t none = 4u * (uint32_t)f.nq;  // counted in the extra word, matched by no group
+    if (t < 256) {
+      const uint32_t e = __ldg(f.lut + t);
+      s_lut[t] = (uint8_t)((e >> 3) < (uint32_t)f.B ? e >> 3 : none);
+    }
+    __syncthreads();
+  }
+  const uint32_t mine = smem_u32(hist + t);
+  auto count = [&](uint32_t v) { bump_byte(mine + v + (v >> 2) * (kCountThreads * 4 - 4)); };
+  auto clear = [&]() {
+    for (int e = t; e < (f.nq + 1) * (kCountThreads / 4); e += kCountThreads)
+      reinterpret_cast<uint4 *>(hist)[e] = make_uint4(0u, 0u, 0u, 0u);
+  };
+  if (blockIdx.z == 0) {
+    const int hc = blockIdx.x;
+    const int y0 = blockIdx.y * col_tile_rows(f), nrows = min(col_tile_rows(f), f.H - y0);
+    const int x4 = hc * kHalf + 4 * (t & 15);
+    const int tcol = (t >> 4) * (kColPitch / 4) + (t & 15);
+    constexpr int kRowStep = kCountThreads / 16, kTileStep = kRowStep * (kColPitch / 4);
+    load_tile<MODE>(f, s_lut, y0, t >> 4, kRowStep, nrows, x4, tile32 + tcol, kTileStep, !f.early);
+    clear();
+    if (f.early) {
+      griddep_wait();
+      const uint32_t *rp = tile32 + tcol;
+      uint8_t *qp = f.q + (size_t)(y0 + (t >> 4)) * wpad + x4;
+      for (int r = t >> 4; r < nrows; r += kRowStep, rp += kTileStep, qp += kRowStep * wpad)
+        *reinterpret_cast<uint32_t *>(qp) = *rp;
+    }
+    __syncthreads();
+    const int x = t & (kHalf - 1), piece = t / kHalf;
+    {
+      const int n = max(0, min(per, nrows - piece * per));
+      const uint8_t *col = smem_raw + piece * per * kColPitch + x;
+      int r = 0;
+      for (; r + 4 <= n; r += 4) {
+        uint32_t v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = col[(r + i) * kColPitch];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) count(v[i]);
+      }
+      for (; r < n; ++r) count(col[r * kColPitch]);
+    }
+    __syncthreads();
+    // thread (column, every eighth group): down each superband's bands
+    const size_t band_step = (size_t)f.nq * wpad;
+    const int sb0 = blockIdx.y << 1 >> f.split, sb1 = min(sb0 + (2 >> f.split), f.nsb);
+    for (int g = piece; g < f.nq; g += kCountThreads / kHalf) {
+      const uint32_t *hg = hist + g * kCountThreads + x;
+      const size_t at = (size_t)g * wpad + hc * kHalf + x;
+      for (int sb = sb0; sb < sb1; ++sb) {
+        uint32_t *pb = f.pb + (size_t)sb * kSuper * band_step + at;
+        uint32_t above[kSuper + 1];  // bytes of at most 4R <= 128
+        above[0] = 0u;
+#pragma unroll
+        for (int j = 0; j < kSuper; ++j) {
+          above[j + 1] = above[j] + hg[0];
+          if (f.split) above[j + 1] += hg[kHalf];
+          hg += kHalf << f.split;
+        }
+        const int nbk = f.nbands - sb * kSuper;
+#pragma unroll
+        for (int j = 1; j < kSuper; ++j) {
+          pb += band_step;
+          if (j < nbk) *pb = above[j];
+        }
+        f.sb[(size_t)sb * band_step + at] = above[kSuper];
+      }
+    }
+  } else {
+    const int c = blockIdx.x >> 1;
+    const int trows = row_tile_rows(f), lr = __ffs(trows) - 1;
+    const int y0 = (2 * blockIdx.y + (blockIdx.x & 1)) * trows, nrows = min(trows, f.H - y0);
+    load_tile<MODE>(f, s_lut, y0, w, kCountThreads / 32, nrows, c * kChunk + 4 * lane,
+                    tile32 + w * (kRowPitch / 4) + lane, kCountThreads / 32 * (kRowPitch / 4), false);
+    clear();
+    if (f.early) griddep_wait();
+    __syncthreads();
+    const int r = t & (trows - 1), piece = t >> lr, pieces = kCountThreads >> lr;
+    if (r < nrows) {
+      const uint32_t *src = tile32 + r * (kRowPitch / 4) + piece * (per / 4);
+#pragma unroll 2
+      for (int i = 0; i < per / 4; ++i) {
+        const uint32_t v = src[i];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) count(__byte_perm(v, 0u, 0x4440u + e));
+      }
+    }
+    __syncthreads();
+    const size_t hpad = (size_t)f.nsb * kSuper * f.R;
+    if (y0 < (int)hpad) {
+      // thread (row, every pieces-th group); a warp may hold two groups
+      const uint32_t *hg = hist + piece * kCountThreads + r;
+      uint32_t *rl = f.rl + ((size_t)c * f.nq + piece) * hpad + y0 + r;
+      const int y = y0 + r;
+      const int k = y >> (__ffs(f.R) - 1);
+      const bool first = (y & (f.R - 1)) == 0 && y < f.H;
+      uint2 *ct = f.ct + ((size_t)k * f.nq + piece) * f.nchunks + c;
+      for (int g0 = 0; g0 < f.nq; g0 += pieces) {
+        const bool in = g0 + piece < f.nq;
+        uint32_t n = 0u;  // bytes of at most 128
+        if (in) {
+#pragma unroll 4
+          for (int p = 0; p < kCountThreads; p += trows) n += hg[p];
+          *rl = n;
+        }
+        if (f.nsegs > 1) {
+          // a band's R rows lie in neighbouring lanes
+          uint32_t lo = n & 0x00ff00ffu, hi = (n >> 8) & 0x00ff00ffu;
+          if (f.R == 32) {
+            lo = __reduce_add_sync(kFull, lo);
+            hi = __reduce_add_sync(kFull, hi);
+          } else {
+            for (int d = 1; d < f.R; d <<= 1) {
+              lo += __shfl_xor_sync(kFull, lo, d);
+              hi += __shfl_xor_sync(kFull, hi, d);
+            }
+          }
+          if (in && first) *ct = make_uint2(lo, hi);
+          ct += (size_t)pieces * f.nchunks;
+        }
+        hg += pieces * kCountThreads;
+        rl += (size_t)pieces * hpad;
+      }
+    }
+  }
+  griddep_release();
+}
+
+// Inclusive prefix of v[0..3] (this lane's 4 columns) over the chunk.
+__device__ __forceinline__ void chunk_prefix(uint32_t v[4], int lane) {
+  v[1] += v[0];
+  v[2] += v[1];
+  v[3] += v[2];
+  const uint32_t s = warp_scan_incl(v[3], lane);
+  const uint32_t ex = s - v[3];
+  v[0] += ex;
+  v[1] += ex;
+  v[2] += ex;
+  v[3] = s;
+}
+
+__device__ __forceinline__ void add_bytes16(uint32_t &lo, uint32_t &hi, uint32_t w) {
+  lo += w & 0x00ff00ffu;         // bins 0 and 2
+  hi += (w >> 8) & 0x00ff00ffu;  // bins 1 and 3
+}
+
+// One CTA per (band, group, width segment), one warp per chunk of the
+// segment.  LAYOUT: 0 bin-major, 2 quad-major.  VEC: rows of H (quad-major:
+// its 16-byte words) start on 16-byte boundaries.  Bin-major rows that do not
+// (W no multiple of 4) leave as 4-byte stores, 128 contiguous bytes each:
+// after the scan the lanes exchange columns through shared memory, from 4
+// neighbouring ones per lane to columns lane, lane + 32, .. -- one word per
+// column for the four bins, so the exchange costs 5 accesses a row.
+template <int LAYOUT, bool VEC>
+__global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4) band_emit_kernel(const __grid_constant__ BandDesc f) {
+  __shared__ uint4 s_row[kSegWarps][32];   // per chunk: counts left of it, per row of the band
+  __shared__ uint2 s_own[kSegWarps][32];   // per chunk: its own counts, per row (16-bit lanes)
+  __shared__ uint2 s_left[kSegWarps][32];  // per warp: its share of the chunks left of the segment
+  __shared__ uint4 s_tot[kSegWarps];       // per chunk: its counts in the rows above the band
+  __shared__ uint4 s_ltot[kSegWarps];      // per warp: its share of the same left of the segment
+  constexpr bool SPREAD = LAYOUT == 0 && !VEC;
+  constexpr int P = 4;  // rows in hand at a time
+  __shared__ __align__(16) uint32_t s_col[SPREAD ? kSegWarps : 1][SPREAD ? 4 : 1][SPREAD ? kChunk : 4];
+  griddep_wait();
+  griddep_release();
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  unsigned int it = blockIdx.x;
+  const int seg = (int)(it % (unsigned)f.nsegs);
+  it /= (unsigned)f.nsegs;
+  const int g = (int)(it % (unsigned)f.nq);
+  const int k = (int)(it / (unsigned)f.nq);
+  const int c0 = seg * f.cps;
+  const int c = c0 + w;
+  const bool live = c < f.nchunks;
+  const int y0 = k * f.R;
+  const int nrows = min(f.R, f.H - y0);
+  const size_t wpad = (size_t)f.nchunks * kChunk;
+  const size_t hpad = (size_t)f.nsb * kSuper * f.R;
+  const int sbk = k / kSuper;
+  const int x = c * kChunk + 4 * lane;
+  const uint8_t *qp = f.q + (size_t)y0 * wpad + x;
+  uint32_t px[P];
+  uint32_t acc[4][4];  // running H of this lane's 4 columns, per bin
+  if (live) {
+#pragma unroll
+    for (int i = 0; i < P; ++i) px[i] = i < nrows ? __ldcg(reinterpret_cast<const unsigned int *>(qp + (size_t)i * wpad)) : 0u;
+    const uint32_t own = lane < f.R ? __ldcg(f.rl + ((size_t)c * f.nq + g) * hpad + y0 + lane) : 0u;
+    // counts above the band in this lane's columns, two bins per word
+    uint32_t lo[4], hi[4];
+    {
+      const uint4 p = k % kSuper ? __ldcg(reinterpret_cast<const uint4 *>(f.pb + ((size_t)k * f.nq + g) * wpad + x))
+                                 : make_uint4(0u, 0u, 0u, 0u);  // a superband's first band
+      const uint32_t pv[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        lo[i] = hi[i] = 0u;
+        add_bytes16(lo[i], hi[i], pv[i]);
+      }
+    }
+    const uint32_t *sp = f.sb + (size_t)g * wpad + x;
+    const size_t sstep = (size_t)f.nq * wpad;
+#pragma unroll 4
+    for (int s = 0; s < sbk; ++s) {
+      const uint4 p = __ldcg(reinterpret_cast<const uint4 *>(sp + s * sstep));
+      add_bytes16(lo[0], hi[0], p.x);
+      add_bytes16(lo[1], hi[1], p.y);
+      add_bytes16(lo[2], hi[2], p.z);
+      add_bytes16(lo[3], hi[3], p.w);
+    }
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[b][i] = (((b & 1) ? hi[i] : lo[i]) >> (b & 2 ? 16 : 0)) & 0xffffu;
+      chunk_prefix(acc[b], lane);
+    }
+    if (lane == 31) s_tot[w] = make_uint4(acc[0][3], acc[1][3], acc[2][3], acc[3][3]);
+    uint2 o = make_uint2(0u, 0u);
+    add_bytes16(o.x, o.y, own);
+    s_own[w][lane] = o;
+  }
+  if (seg > 0) {
+    // the chunks left of the segment, shared out over the CTA's warps
+    uint2 l = make_uint2(0u, 0u);
+    for (int cl = w; cl < c0; cl += nw)
+      if (lane < f.R) add_bytes16(l.x, l.y, __ldcg(f.rl + ((size_t)cl * f.nq + g) * hpad + y0 + lane));
+    s_left[w][lane] = l;
+    uint4 tot = make_uint4(0u, 0u, 0u, 0u);
+    auto add = [&](uint2 v) {
+      tot.x += v.x & 0xffffu;
+      tot.z += v.x >> 16;
+      tot.y += v.y & 0xffffu;
+      tot.w += v.y >> 16;
+    };
+    for (int e = threadIdx.x; e < k * c0; e += blockDim.x) {
+      const int j = e / c0, cl = e - j * c0;
+      add(__ldcg(f.ct + ((size_t)j * f.nq + g) * f.nchunks + cl));
+    }
+    tot.x = __reduce_add_sync(kFull, tot.x);
+    tot.y = __reduce_add_sync(kFull, tot.y);
+    tot.z = __reduce_add_sync(kFull, tot.z);
+    tot.w = __reduce_add_sync(kFull, tot.w);
+    if (lane == 0) s_ltot[w] = tot;
+  }
+  __syncthreads();
+  if (!live) return;
+  {
+    uint4 l = make_uint4(0u, 0u, 0u, 0u);
+    uint2 r = make_uint2(0u, 0u);
+    for (int i = 0; i < w; ++i) {
+      const uint4 v = s_tot[i];
+      l.x += v.x; l.y += v.y; l.z += v.z; l.w += v.w;
+      const uint2 o = s_own[i][lane];
+      r.x += o.x; r.y += o.y;
+    }
+    if (seg > 0)
+      for (int i = 0; i < nw; ++i) {
+        const uint4 v = s_ltot[i];
+        l.x += v.x; l.y += v.y; l.z += v.z; l.w += v.w;
+        const uint2 o = s_left[i][lane];
+        r.x += o.x; r.y += o.y;
+      }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      acc[0][i] += l.x; acc[1][i] += l.y; acc[2][i] += l.z; acc[3][i] += l.w;
+    }
+    s_row[w][lane] = make_uint4(r.x & 0xffffu, r.y & 0xffffu, r.x >> 16, r.y >> 16);
+    __syncwarp();
+  }
+  const uint32_t gbase = 32u * (uint32_t)g;
+  const size_t plane = (size_t)f.H * (size_t)f.W;
+  const int nb = min(4, f.B - 4 * g);
+  const uint32_t *out_end = f.out + plane * (size_t)f.B;
+  (void)out_end;
+  // element e of this lane: column x + e, or column c * 128 + lane + 32 e
+  const int xs = SPREAD ? c * kChunk + lane : x;
+  if constexpr (SPREAD) {
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      *reinterpret_cast<uint4 *>(&s_col[w][b][4 * lane]) = make_uint4(acc[b][0], acc[b][1], acc[b][2], acc[b][3]);
+    __syncwarp();
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[b][e] = s_col[w][b][32 * e + lane];
+    __syncwarp();
+  }
+  uint32_t *o = LAYOUT == 0 ? f.out + ((size_t)(4 * g) * f.H + y0) * f.W + xs
+                            : f.out + (((size_t)g * f.H + y0) * f.W + x) * 4;
+  for (int r0 = 0; r0 < nrows; r0 += P) {
+    // the prefix of P rows' one-hot bytes along the chunk, four bins to a
+    // word; the rows' shuffles are independent
+    uint32_t p[P][4], tot[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) p[i][e] = shl_clamp(1u, 8u * __byte_perm(px[i], 0u, 0x4440u + e) - gbase);
+      p[i][1] += p[i][0];
+      p[i][2] += p[i][1];
+      p[i][3] += p[i][2];
+      tot[i] = p[i][3];
+    }
+    qp += (size_t)P * wpad;
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+      px[i] = r0 + P + i < nrows ? __ldcg(reinterpret_cast<const unsigned int *>(qp + (size_t)i * wpad)) : 0u;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      uint32_t n[P];
+#pragma unroll
+      for (int i = 0; i < P; ++i) n[i] = __shfl_up_sync(kFull, tot[i], d);
+#pragma unroll
+      for (int i = 0; i < P; ++i)
+        if (lane >= d) tot[i] += n[i];  // bytes of at most 128
+    }
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+      const uint32_t ex = tot[i] - p[i][3];
+      p[i][0] += ex;
+      p[i][1] += ex;
+      p[i][2] += ex;
+      p[i][3] = tot[i];
+    }
+    if constexpr (SPREAD) {
+#pragma unroll
+      for (int i = 0; i < P; ++i)
+        *reinterpret_cast<uint4 *>(&s_col[w][i][4 * lane]) = make_uint4(p[i][0], p[i][1], p[i][2], p[i][3]);
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < P; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) p[i][e] = s_col[w][i][32 * e + lane];
+      __syncwarp();
+    }
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+      if (r0 + i >= nrows) break;
+      const uint4 rc = s_row[w][r0 + i];
+      const uint32_t rcv[4] = {rc.x, rc.y, rc.z, rc.w};
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[b][e] += __byte_perm(p[i][e], 0u, 0x4440u + b) + rcv[b];
+      if constexpr (LAYOUT == 0) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          if (b < nb) {
+            uint32_t *ob = o + b * plane;
+            if (VEC) {
+              if (x < f.W && IHIST_GUARD(f.ctrl, ob >= f.out && ob + 4 <= out_end)) st_stream_v4(ob, acc[b][0], acc[b][1], acc[b][2], acc[b][3]);
+            } else {
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                if (xs + 32 * e < f.W && IHIST_GUARD(f.ctrl, ob + 32 * e >= f.out && ob + 32 * e < out_end))
+                  st_stream(ob + 32 * e, acc[b][e]);
+            }
+          }
+        }
+        o += f.W;
+      } else {
+        const bool v8 = VEC && (reinterpret_cast<uintptr_t>(o) & 31u) == 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const uint4 a0 = make_uint4(acc[0][2 * h], acc[1][2 * h], acc[2][2 * h], acc[3][2 * h]);
+          const uint4 a1 = make_uint4(acc[0][2 * h + 1], acc[1][2 * h + 1], acc[2][2 * h + 1], acc[3][2 * h + 1]);
+          if (v8 && x + 2 * h + 1 < f.W) {
+            if (IHIST_GUARD(f.ctrl, o + 8 * h >= f.out && o + 8 * h + 8 <= out_end)) st_stream_v8(o + 8 * h, a0, a1);
+          } else {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const uint4 v = e ? a1 : a0;
+              uint32_t *oe = o + 8 * h + 4 * e;
+              if (x + 2 * h + e < f.W && IHIST_GUARD(f.ctrl, oe >= f.out && oe + 4 <= out_end)) {
+                if (VEC) {
+                  st_stream_v4(oe, v.x, v.y, v.z, v.w);
+                } else {
+                  st_stream(oe, v.x);
+                  st_stream(oe + 1, v.y);
+                  st_stream(oe + 2, v.z);
+                  st_stream(oe + 3, v.w);
+                }
+              }
+            }
+          }
+        }
+        o += (size_t)f.W * 4;
+      }
+    }
+  }
+}
+
+}  // namespace ihist
