@@ -250,20 +250,21 @@ int ihist_query(ihist_plan_t plan, const uint32_t *d_hist, const int32_t *d_rect
  * H, with the corner lookups put in row order first (same results as
  * ihist_query, word for word).  ihist_query reads each corner word where it
  * lies, so random rectangles on a large bin-major H cost one DRAM line per
- * 4-byte corner; here the corners of all n rectangles are bucketed by row
- * (a counting sort, once per call), then each group of bins_per_pass bins
- * reads them bucket by bucket, so the corners of a row share the lines they
- * fall on, and a second pass combines each rectangle's four corners.
+ * 4-byte corner; here the corner pairs (x1, x0-1) of each rectangle's two
+ * rows are bucketed by row (a counting sort, once per call), then each group
+ * of bins_per_pass bins reads them bucket by bucket, so the corners of a row
+ * share the lines they fall on, and a second pass subtracts each rectangle's
+ * upper row from its lower one.
  *   bins_per_pass  bins gathered per pass: 4, 8 or 16 (0 = 8)
  *   d_work         device scratch of ihist_query_work_bytes(plan, n,
  *                  bins_per_pass) bytes, 256-byte aligned, owned by the
- *                  caller; about 32 + 16 * bins_per_pass bytes per rectangle
+ *                  caller; about 24 + 8 * bins_per_pass bytes per rectangle
  *                  plus 8 per frame row.  Its contents need not be kept
  *                  between calls; two calls sharing it must not overlap.
  * Other arguments and the bad-rectangle rule as for ihist_query.  Bin-major
  * plans only (IHIST_ERR_UNSUPPORTED otherwise); n < 2^29;
  * IHIST_ERR_INVALID_ARG if work_bytes is too small.  Five kinds of launch on
- * `stream` (count, offsets, scatter, then a gather and a combine per group
+ * `stream` (rank, offsets, scatter, then a gather and a combine per group
  * of bins); allocates nothing. */
 size_t ihist_query_work_bytes(ihist_plan_t plan, int n, int bins_per_pass);
 int ihist_query_sorted(ihist_plan_t plan, const uint32_t *d_hist, const int32_t *d_rects, int n,

@@ -788,9 +788,9 @@ extern "C" int ihist_query(ihist_plan_t p, const uint32_t *d_hist, const int32_t
                       stream);
 }
 
-// Scratch of ihist_query_sorted: row counts (zero between calls), row
-// offsets, the corners' (y, x) in row order, each rectangle's four corner
-// positions and the gathered corner values of one bin group.
+// Scratch of ihist_query_sorted: row counts, row offsets, the row pairs in
+// row order, each rectangle's two pair positions and the differences of one
+// bin group.
 struct SortedQueryWork {
   size_t o_cnt, o_off, o_pts, o_slot, o_val, bytes;
 };
@@ -803,13 +803,29 @@ static SortedQueryWork sorted_query_work(int H, size_t n, int nb) {
   w.o_off = off;
   off = align_up(off + ((size_t)H + 1) * 4, 256);
   w.o_pts = off;
-  off = align_up(off + 4 * n * 4, 256);
+  off = align_up(off + 2 * n * 8, 256);
   w.o_slot = off;
-  off = align_up(off + n * 16, 256);
+  off = align_up(off + n * 8, 256);
   w.o_val = off;
-  off = align_up(off + 4 * n * (size_t)nb * 4, 256);
+  off = align_up(off + 2 * n * (size_t)nb * 4, 256);
   w.bytes = off;
   return w;
+}
+
+// Gather and combine of one group of NB bins (nb of them present).
+template <int NB>
+static void launch_sorted_group(const uint32_t *hist, int H, int W, int B, int b0, int nb, const uint2 *pts,
+                                const unsigned int *off, const uint2 *slot, unsigned int n, uint32_t *val,
+                                uint32_t *out, unsigned int cap, cudaStream_t s) {
+  constexpr unsigned int gt = gather_threads(NB);
+  const unsigned int g_pair = (2u * n + gt - 1u) / gt;  // n < 2^29
+  const unsigned int g_comb =
+      (unsigned int)std::min<unsigned long long>(((unsigned long long)n * (NB / 4) + 255ull) / 256ull, cap);
+  pair_gather_kernel<NB><<<g_pair, gt, 0, s>>>(hist, H, W, b0, nb, pts, off, val);
+  if (nb == NB && B % 4 == 0 && ((uintptr_t)out & 15u) == 0)
+    pair_combine_kernel<NB, true><<<g_comb, 256, 0, s>>>(slot, n, B, b0, nb, val, out);
+  else
+    pair_combine_kernel<NB, false><<<g_comb, 256, 0, s>>>(slot, n, B, b0, nb, val, out);
 }
 
 static int sorted_group(int bins_per_pass) { return bins_per_pass == 0 ? 8 : bins_per_pass; }
@@ -842,34 +858,28 @@ extern "C" int ihist_query_sorted(ihist_plan_t p, const uint32_t *d_hist, const 
   char *base = static_cast<char *>(d_work);
   unsigned int *cnt = reinterpret_cast<unsigned int *>(base + w.o_cnt);
   unsigned int *off = reinterpret_cast<unsigned int *>(base + w.o_off);
-  uint32_t *pts = reinterpret_cast<uint32_t *>(base + w.o_pts);
-  uint4 *slot = reinterpret_cast<uint4 *>(base + w.o_slot);
+  uint2 *pts = reinterpret_cast<uint2 *>(base + w.o_pts);
+  uint2 *slot = reinterpret_cast<uint2 *>(base + w.o_slot);
   uint32_t *val = reinterpret_cast<uint32_t *>(base + w.o_val);
   cudaStream_t s = (cudaStream_t)stream;
   const unsigned int un = (unsigned int)n;
   const unsigned int cap = (unsigned int)p->sms * 16u;
   const unsigned int g_rect = std::min<unsigned int>((un + 255u) / 256u, cap);
-  const unsigned int g_pts = std::min<unsigned int>((unsigned int)(((unsigned long long)un * 4ull + 255ull) / 256ull), cap);
   if (cudaMemsetAsync(cnt, 0, (size_t)p->H * 4, s) != cudaSuccess) return IHIST_ERR_CUDA;
-  corner_count_kernel<<<g_rect, 256, 0, s>>>(d_rects, un, p->H, p->W, cnt, p->ctrl);
+  pair_rank_kernel<<<g_rect, 256, 0, s>>>(d_rects, un, p->H, p->W, cnt, slot, p->ctrl);
   row_offsets_kernel<<<1, 1024, 0, s>>>(cnt, p->H, off);
-  corner_scatter_kernel<<<g_rect, 256, 0, s>>>(d_rects, un, p->H, p->W, cnt, off, pts, slot);
+  pair_scatter_kernel<<<g_rect, 256, 0, s>>>(d_rects, un, p->H, p->W, off, pts, slot);
   for (int b0 = 0; b0 < p->B; b0 += nb) {
     const int cur = std::min(nb, p->B - b0);
-    const unsigned int g_comb = std::min<unsigned int>(
-        (unsigned int)(((unsigned long long)un * nb + 255ull) / 256ull), cap);
     switch (nb) {
       case 4:
-        corner_gather_kernel<4><<<g_pts, 256, 0, s>>>(d_hist, p->H, p->W, b0, cur, pts, off, val);
-        corner_combine_kernel<4><<<g_comb, 256, 0, s>>>(slot, un, p->B, b0, cur, val, d_hist_out);
+        launch_sorted_group<4>(d_hist, p->H, p->W, p->B, b0, cur, pts, off, slot, un, val, d_hist_out, cap, s);
         break;
       case 8:
-        corner_gather_kernel<8><<<g_pts, 256, 0, s>>>(d_hist, p->H, p->W, b0, cur, pts, off, val);
-        corner_combine_kernel<8><<<g_comb, 256, 0, s>>>(slot, un, p->B, b0, cur, val, d_hist_out);
+        launch_sorted_group<8>(d_hist, p->H, p->W, p->B, b0, cur, pts, off, slot, un, val, d_hist_out, cap, s);
         break;
       default:
-        corner_gather_kernel<16><<<g_pts, 256, 0, s>>>(d_hist, p->H, p->W, b0, cur, pts, off, val);
-        corner_combine_kernel<16><<<g_comb, 256, 0, s>>>(slot, un, p->B, b0, cur, val, d_hist_out);
+        launch_sorted_group<16>(d_hist, p->H, p->W, p->B, b0, cur, pts, off, slot, un, val, d_hist_out, cap, s);
         break;
     }
   }

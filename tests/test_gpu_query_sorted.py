@@ -83,3 +83,27 @@ def test_sorted_query_argument_checks():
             assert e.value.code == ihist.IHIST_ERR_INVALID_ARG
         ihist.ihist_query_sorted(plan.handle, out.data_ptr(), rects.data_ptr(), 0, res.data_ptr(), 0, 0, 0)
         assert plan.query_work_bytes(100, 5) == 0
+
+
+@pytest.mark.parametrize("bpp", [4, 8, 16])
+@pytest.mark.parametrize("nbins", [5, 16, 18])
+def test_sorted_query_row_pairs(nbins, bpp):
+    """Rectangles whose pairs lack a row (y0 = 0), a column (x0 = 0) or both,
+    many in one row, more pairs than one CTA of the gather, an output that is
+    not 16-byte aligned, and a partial last group."""
+    h, w = 40, 300
+    img = synth.uniform_frame(17, h, w)
+    base = synth.rects(23, 600, h, w)
+    left, top, row = base.copy(), base.copy(), base.copy()
+    left[:, 0], top[:, 1] = 0, 0
+    row[:, 1], row[:, 3] = 7, 7
+    rects = np.concatenate([base, left, top, row, np.minimum(left, top), edge_rects(h, w)])
+    ref = oracle.query(oracle.integral_histogram(img, nbins), rects)
+    with ihist.Plan(h, w, nbins) as plan:
+        hist = plan.compute(torch.from_numpy(img).cuda())
+        buf = torch.full((1 + len(rects) * nbins + 8,), -3, dtype=torch.int32, device="cuda")
+        out = buf[1:1 + len(rects) * nbins].view(len(rects), nbins)
+        plan.query_sorted(hist, torch.from_numpy(rects).cuda(), out=out, bins_per_pass=bpp)
+        assert plan.status() == ihist.IHIST_OK
+    assert np.array_equal(out.cpu().numpy().view(np.uint32), ref)
+    assert int(buf[0]) == -3 and bool((buf[1 + len(rects) * nbins:] == -3).all())
