@@ -73,7 +73,7 @@ typedef struct ihist_plan_s *ihist_plan_t;
  * default for the frame shape.  A plan that leaves every tiling field zero
  * (rows_per_band, bins_per_cta, chunks_per_warp, groups_per_cta, ctas_per_sm,
  * warps_per_cta) may take the two-launch path instead (a count kernel, then
- * an emit kernel; bin- and quad-major frames up to 12 and 40 megapixels),
+ * an emit kernel; bin-major frames up to 12 megapixels, others up to 40),
  * which has no tiling of its own: ihist_plan_get_tune then reports the tiling
  * of the fused kernel for the shape, and passing it back selects that kernel.
  * Results are the same words either way.

@@ -395,7 +395,7 @@ static int plan_create(int h, int w, int nbins, int layout, const ihist_tune_t *
       delete p;
       return IHIST_ERR_CUDA;
     }
-    const int brc = bands_prepare(band, mode, (size_t)optin_b);
+    const int brc = bands_prepare(band, mode, layout, (size_t)optin_b);
     if (brc == IHIST_ERR_UNSUPPORTED) {
       banded = false;
     } else if (brc != IHIST_OK) {

@@ -13,7 +13,9 @@
 // pixels, GB300): 320x240 x 16 16.9 -> 6.2 us, 640x480 x 32 21.4 -> 11.4,
 // 1280x720 x 32 36 -> 26, 1920x1080 x 64 104.9 -> 85.5 (a plain fill of the
 // same bytes takes 78.5), 1921x1081 x 64 160 -> 92, 3840x2160 x 64 355 -> 329;
-// quad-major 1920x1080 x 64 108 -> 90, 1921x1081 x 64 582 -> 116.
+// quad-major 1920x1080 x 64 108 -> 90, 1921x1081 x 64 582 -> 116; pixel-major
+// 640x480 x 64 61 -> 24, 1920x1080 x 64 150 -> 95, 1921x1081 x 37 300 -> 77,
+// 3840x2160 x 64 521 -> 350.
 //
 // Superband: 4 bands of R rows (R = 8, 16 or 32).  A group is 4 bins, packed
 // as the bytes of one word; a chunk is 128 columns.  The count kernel leaves
@@ -22,7 +24,9 @@
 //                                    this one within its superband (bytes)
 //   sb   [superband][group][column]  counts of the column in the superband
 //   rl   [chunk][group][row]         counts of the row inside the chunk
-//   ct   [band][group][chunk]        counts of the band inside the chunk
+//   rls  [chunk][3][group][row]      counts of the row inside the chunk's first
+//                                    32, 64 and 96 columns (pixel-major only)
+//   ct   [group][chunk][band]        counts of the band inside the chunk
 //                                    (16-bit lanes; only when a band is split
 //                                    into width segments)
 // and a band's first row of H follows from pb, the sb above and a scan along
@@ -51,13 +55,20 @@ struct BandDesc {
   int R, nbands, nsb, nq, nchunks, nsegs, cps;
   int split;  // a count thread counts R >> split pixels
   uint8_t *q;
-  uint32_t *pb, *sb, *rl;
+  int bpb, nblk;  // pixel-major: bins of one CTA (a multiple of 4, at most 64) and blocks of them
+  uint32_t *pb, *sb, *rl, *rls;
   uint2 *ct;
   Ctrl *ctrl;  // checked builds: where a failed store check is latched
 };
 
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// 16 bytes from global to shared memory, past L1 (both addresses aligned).
+__device__ __forceinline__ void copy_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // One more in a byte counter of this thread's own (shared memory address).
 __device__ __forceinline__ void bump_byte(uint32_t a) {
@@ -268,13 +279,25 @@ __global__ void __launch_bounds__(kCountThreads, 4) band_count_kernel(const __gr
       const int y = y0 + r;
       const int k = y >> (__ffs(f.R) - 1);
       const bool first = (y & (f.R - 1)) == 0 && y < f.H;
-      uint2 *ct = f.ct + ((size_t)k * f.nq + piece) * f.nchunks + c;
+      uint2 *ct = f.ct + ((size_t)piece * f.nchunks + c) * f.nbands + k;
       for (int g0 = 0; g0 < f.nq; g0 += pieces) {
         const bool in = g0 + piece < f.nq;
         uint32_t n = 0u;  // bytes of at most 128
         if (in) {
+          if (f.rls == nullptr) {
 #pragma unroll 4
-          for (int p = 0; p < kCountThreads; p += trows) n += hg[p];
+            for (int p = 0; p < kCountThreads; p += trows) n += hg[p];
+          } else {
+            const int strip = (kCountThreads / 4) - 1;  // a quarter of the pieces, each trows counters
+            uint32_t *rls = f.rls + ((size_t)(3 * c) * f.nq + g0 + piece) * hpad + y0 + r;
+            for (int p = 0; p < kCountThreads; p += trows) {
+              n += hg[p];
+              if (((p + trows) & strip) == 0 && p + trows < kCountThreads) {
+                *rls = n;
+                rls += (size_t)f.nq * hpad;
+              }
+            }
+          }
           *rl = n;
         }
         if (f.nsegs > 1) {
@@ -290,7 +313,7 @@ __global__ void __launch_bounds__(kCountThreads, 4) band_count_kernel(const __gr
             }
           }
           if (in && first) *ct = make_uint2(lo, hi);
-          ct += (size_t)pieces * f.nchunks;
+          ct += (size_t)pieces * f.nchunks * f.nbands;
         }
         hg += pieces * kCountThreads;
         rl += (size_t)pieces * hpad;
@@ -318,6 +341,9 @@ __device__ __forceinline__ void add_bytes16(uint32_t &lo, uint32_t &hi, uint32_t
   hi += (w >> 8) & 0x00ff00ffu;  // bins 1 and 3
 }
 
+// Dynamic shared memory of the emit kernel: the band's bins.
+__host__ __device__ inline size_t emit_smem_bytes(int warps, int R) { return (size_t)warps * R * kChunk; }
+
 // One CTA per (band, group, width segment), one warp per chunk of the
 // segment.  LAYOUT: 0 bin-major, 2 quad-major.  VEC: rows of H (quad-major:
 // its 16-byte words) start on 16-byte boundaries.  Bin-major rows that do not
@@ -335,6 +361,7 @@ __global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4) b
   constexpr bool SPREAD = LAYOUT == 0 && !VEC;
   constexpr int P = 4;  // rows in hand at a time
   __shared__ __align__(16) uint32_t s_col[SPREAD ? kSegWarps : 1][SPREAD ? 4 : 1][SPREAD ? kChunk : 4];
+  extern __shared__ __align__(16) uint8_t smem_raw[];  // per chunk: the band's bins, R rows of 128 bytes
   griddep_wait();
   griddep_release();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -352,12 +379,12 @@ __global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4) b
   const size_t hpad = (size_t)f.nsb * kSuper * f.R;
   const int sbk = k / kSuper;
   const int x = c * kChunk + 4 * lane;
-  const uint8_t *qp = f.q + (size_t)y0 * wpad + x;
-  uint32_t px[P];
+  uint8_t *tile = smem_raw + (size_t)w * f.R * kChunk;
   uint32_t acc[4][4];  // running H of this lane's 4 columns, per bin
   if (live) {
-#pragma unroll
-    for (int i = 0; i < P; ++i) px[i] = i < nrows ? __ldcg(reinterpret_cast<const unsigned int *>(qp + (size_t)i * wpad)) : 0u;
+    const uint8_t *qp = f.q + (size_t)y0 * wpad + c * kChunk;
+    for (int r = lane >> 3; r < nrows; r += 4)
+      copy_async16(tile + r * kChunk + 16 * (lane & 7), qp + (size_t)r * wpad + 16 * (lane & 7));
     const uint32_t own = lane < f.R ? __ldcg(f.rl + ((size_t)c * f.nq + g) * hpad + y0 + lane) : 0u;
     // counts above the band in this lane's columns, two bins per word
     uint32_t lo[4], hi[4];
@@ -405,16 +432,16 @@ __global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4) b
       tot.y += v.y & 0xffffu;
       tot.w += v.y >> 16;
     };
-    for (int e = threadIdx.x; e < k * c0; e += blockDim.x) {
-      const int j = e / c0, cl = e - j * c0;
-      add(__ldcg(f.ct + ((size_t)j * f.nq + g) * f.nchunks + cl));
-    }
+#pragma unroll 4
+    for (int cl = w; cl < c0; cl += nw)
+      for (int j = lane; j < k; j += 32) add(__ldcg(f.ct + ((size_t)g * f.nchunks + cl) * f.nbands + j));
     tot.x = __reduce_add_sync(kFull, tot.x);
     tot.y = __reduce_add_sync(kFull, tot.y);
     tot.z = __reduce_add_sync(kFull, tot.z);
     tot.w = __reduce_add_sync(kFull, tot.w);
     if (lane == 0) s_ltot[w] = tot;
   }
+  copy_async_wait();
   __syncthreads();
   if (!live) return;
   {
@@ -466,17 +493,15 @@ __global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4) b
     uint32_t p[P][4], tot[P];
 #pragma unroll
     for (int i = 0; i < P; ++i) {
+      // R is a multiple of P: rows past the frame hold what the tile held, and are not stored
+      const uint32_t px = *reinterpret_cast<const uint32_t *>(tile + (r0 + i) * kChunk + 4 * lane);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) p[i][e] = shl_clamp(1u, 8u * __byte_perm(px[i], 0u, 0x4440u + e) - gbase);
+      for (int e = 0; e < 4; ++e) p[i][e] = shl_clamp(1u, 8u * __byte_perm(px, 0u, 0x4440u + e) - gbase);
       p[i][1] += p[i][0];
       p[i][2] += p[i][1];
       p[i][3] += p[i][2];
       tot[i] = p[i][3];
     }
-    qp += (size_t)P * wpad;
-#pragma unroll
-    for (int i = 0; i < P; ++i)
-      px[i] = r0 + P + i < nrows ? __ldcg(reinterpret_cast<const unsigned int *>(qp + (size_t)i * wpad)) : 0u;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       uint32_t n[P];
@@ -560,6 +585,172 @@ __global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4) b
       }
     }
   }
+}
+
+// Pixel-major H[y][x][b].  One CTA per (band, block of bins, chunk), one warp
+// per 32 columns of the chunk and 32 * NJ bins of the block; a lane holds NJ
+// bins (32 apart) of all 32 columns, so that a pixel's counts leave as
+// contiguous stores and a row of a chunk as one run.  Walking along the row,
+// a lane keeps its bins' count of the row so far and adds it to the column's
+// running H: a compare, an add and an add per count, with no scan across
+// lanes at all.  One bin per lane makes twice the warps (1920x1080 x 64: 97
+// us against 104), two keep a record that is no multiple of 32 bytes in one
+// warp's hands, whose stores meet in L2 (1921x1081 x 37: 77 against 111).
+constexpr int kPixelBins = 64;                // bins of one CTA at most
+constexpr int kStripCols = 32;
+constexpr size_t kPixelTopBytes = (size_t)kChunk * kPixelBins * 4;
+__host__ __device__ inline size_t pixel_smem_bytes(int R) {
+  return kPixelTopBytes + (size_t)4 * R * kPixelBins * 2 + (size_t)R * kChunk;
+}
+
+// The rows of one strip.  FULL: all 32 columns lie inside the frame.
+template <int NJ, bool FULL>
+__device__ __forceinline__ void emit_strip(const BandDesc &f, uint32_t (&acc)[kStripCols][NJ], const uint32_t (&bin)[NJ],
+                                           const bool (&has)[NJ], const uint2 *s_left, const uint8_t *tile, int y0,
+                                           int nrows, int x0, int ncols, int b0) {
+  constexpr int kUnits = kPixelBins / 4;
+  uint32_t *row = f.out + ((size_t)y0 * f.W + x0) * f.B + b0;
+  const uint32_t *out_end = f.out + (size_t)f.H * f.W * f.B;
+  (void)out_end;
+  for (int y = 0; y < nrows; ++y) {
+    const uint4 q0 = *reinterpret_cast<const uint4 *>(tile + y * kChunk);
+    const uint4 q1 = *reinterpret_cast<const uint4 *>(tile + y * kChunk + 16);
+    const uint32_t qv[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+    uint32_t rc[NJ];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+      rc[j] = reinterpret_cast<const uint16_t *>(s_left + y * kUnits + ((bin[j] >> 2) ^ (y & 15)))[bin[j] & 3];
+    uint32_t *o = row + bin[0];
+#pragma unroll
+    for (int i = 0; i < kStripCols; ++i) {
+      const uint32_t q = __byte_perm(qv[i >> 2], 0u, 0x4440u + (i & 3));
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        if (q == (uint32_t)b0 + bin[j]) ++rc[j];
+        acc[i][j] += rc[j];
+        if ((FULL || i < ncols) && has[j] && IHIST_GUARD(f.ctrl, o + 32 * j >= f.out && o + 32 * j < out_end))
+          st_stream(o + 32 * j, acc[i][j]);
+      }
+      o += f.B;
+    }
+    row += (size_t)f.W * f.B;
+  }
+}
+
+template <int WARPS, int NJ>
+__global__ void __launch_bounds__(WARPS * 32, NJ == 2 ? 4 : 24 / WARPS) band_emit_pixel_kernel(const __grid_constant__ BandDesc f) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  // first rows of H [column][16-byte unit of 4 bins ^ (column / 4 mod 8)], then
+  // the counts left of each strip [strip][row][8-byte unit of 4 bins ^ (row
+  // mod 16)], then the band's bins [row][column]
+  uint4 *s_top = reinterpret_cast<uint4 *>(smem_raw);
+  uint2 *s_left = reinterpret_cast<uint2 *>(smem_raw + kPixelTopBytes);
+  constexpr int kUnits = kPixelBins / 4;
+  griddep_wait();
+  griddep_release();
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  unsigned int it = blockIdx.x;
+  const int c = (int)(it % (unsigned)f.nchunks);
+  it /= (unsigned)f.nchunks;
+  const int blk = (int)(it % (unsigned)f.nblk);
+  const int k = (int)(it / (unsigned)f.nblk);
+  const int b0 = blk * f.bpb, nb = min(f.bpb, f.B - b0);
+  const int g0 = b0 >> 2, ng = (nb + 3) >> 2;
+  const int y0 = k * f.R, nrows = min(f.R, f.H - y0);
+  const size_t wpad = (size_t)f.nchunks * kChunk;
+  const size_t hpad = (size_t)f.nsb * kSuper * f.R;
+  const int lr = __ffs(f.R) - 1;
+  uint8_t *tile = smem_raw + kPixelTopBytes + (size_t)4 * f.R * kPixelBins * 2;
+  for (int e = threadIdx.x; e < nrows * 8; e += blockDim.x)
+    copy_async16(tile + 16 * e, f.q + (size_t)(y0 + (e >> 3)) * wpad + c * kChunk + 16 * (e & 7));
+  // counts left of each strip, per row and bin
+  for (int e = threadIdx.x; e < ng << lr; e += blockDim.x) {
+    const int gi = e >> lr, y = e & (f.R - 1);
+    const uint32_t *p = f.rl + (size_t)(g0 + gi) * hpad + y0 + y;
+    const size_t step = (size_t)f.nq * hpad;
+    uint32_t lo = 0u, hi = 0u;
+#pragma unroll 8
+    for (int cl = 0; cl < c; ++cl) add_bytes16(lo, hi, __ldcg(p + cl * step));
+    const uint32_t *ps = f.rls + ((size_t)(3 * c) * f.nq + g0 + gi) * hpad + y0 + y;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      uint32_t l = lo, h = hi;
+      if (s > 0) add_bytes16(l, h, __ldcg(ps + (s - 1) * step));
+      s_left[(s * f.R + y) * kUnits + (gi ^ (y & 15))] =
+          make_uint2((l & 0xffffu) | h << 16, l >> 16 | (h & 0xffff0000u));
+    }
+  }
+  // H in the row above the band, four bins of the chunk at a time
+  const int sbk = k / kSuper;
+  for (int gi = w; gi < ng; gi += WARPS) {
+    const int g = g0 + gi;
+    const int x = c * kChunk + 4 * lane;
+    uint32_t lo[4] = {0u, 0u, 0u, 0u}, hi[4] = {0u, 0u, 0u, 0u};
+    auto add = [&](uint4 p) {
+      add_bytes16(lo[0], hi[0], p.x);
+      add_bytes16(lo[1], hi[1], p.y);
+      add_bytes16(lo[2], hi[2], p.z);
+      add_bytes16(lo[3], hi[3], p.w);
+    };
+    const uint32_t *sp = f.sb + (size_t)g * wpad + x;
+    const size_t sstep = (size_t)f.nq * wpad;
+#pragma unroll 4
+    for (int s = 0; s < sbk; ++s) add(__ldcg(reinterpret_cast<const uint4 *>(sp + s * sstep)));
+    if (k % kSuper) add(__ldcg(reinterpret_cast<const uint4 *>(f.pb + ((size_t)k * f.nq + g) * wpad + x)));
+    uint32_t left[4] = {0u, 0u, 0u, 0u};
+    const uint2 *ctp = f.ct + (size_t)g * f.nchunks * f.nbands + lane;
+    for (int j = lane; j < k; j += 32, ctp += 32) {
+#pragma unroll 8
+      for (int cl = 0; cl < c; ++cl) {
+        const uint2 v = __ldcg(ctp + (size_t)cl * f.nbands);
+        left[0] += v.x & 0xffffu;
+        left[2] += v.x >> 16;
+        left[1] += v.y & 0xffffu;
+        left[3] += v.y >> 16;
+      }
+    }
+    uint32_t top[4][4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const uint32_t l = __reduce_add_sync(kFull, left[b]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) top[b][i] = (((b & 1) ? hi[i] : lo[i]) >> (b & 2 ? 16 : 0)) & 0xffffu;
+      chunk_prefix(top[b], lane);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) top[b][i] += l;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      s_top[(4 * lane + i) * kUnits + (gi ^ (lane & 7))] = make_uint4(top[0][i], top[1][i], top[2][i], top[3][i]);
+  }
+  copy_async_wait();
+  __syncthreads();
+  const int strip = w & 3;
+  const int x0 = c * kChunk + kStripCols * strip;
+  const int ncols = min(kStripCols, f.W - x0);
+  if (ncols <= 0) return;
+  // this lane's bins within the block; where there is none it follows the first and stores nothing
+  uint32_t bin[NJ];
+  bool has[NJ];
+#pragma unroll
+  for (int j = 0; j < NJ; ++j) {
+    bin[j] = (uint32_t)(32 * NJ * (w >> 2) + lane + 32 * j);
+    has[j] = bin[j] < (uint32_t)nb;
+    if (!has[j]) bin[j] = 0u;
+  }
+  uint32_t acc[kStripCols][NJ];
+#pragma unroll
+  for (int i = 0; i < kStripCols; ++i) {
+    const int x = kStripCols * strip + i;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+      acc[i][j] = reinterpret_cast<const uint32_t *>(s_top + x * kUnits + ((bin[j] >> 2) ^ (x >> 2 & 7)))[bin[j] & 3];
+  }
+  const uint2 *left = s_left + strip * f.R * kUnits;
+  if (ncols == kStripCols)
+    emit_strip<NJ, true>(f, acc, bin, has, left, tile + kStripCols * strip, y0, nrows, x0, ncols, b0);
+  else
+    emit_strip<NJ, false>(f, acc, bin, has, left, tile + kStripCols * strip, y0, nrows, x0, ncols, b0);
 }
 
 }  // namespace ihist

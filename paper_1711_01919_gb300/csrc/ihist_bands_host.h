@@ -15,9 +15,9 @@ bool bands_shape(int h, int w, int nbins, int layout, int sms, BandDesc *f);
 // pointers into it.
 size_t bands_layout(BandDesc *f, char *base);
 
-// Let the count kernel of this binning use its shared memory (optin: the
+// Let the kernels of this binning and layout use their shared memory (optin: the
 // largest a CTA may have).
-int bands_prepare(const BandDesc &f, int mode, size_t optin);
+int bands_prepare(const BandDesc &f, int mode, int layout, size_t optin);
 
 // Both launches, with programmatic stream serialization.
 int launch_bands(const BandDesc &f, int mode, int layout, void *stream);

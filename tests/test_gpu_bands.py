@@ -1,8 +1,8 @@
 """The two-launch path (count kernel, then emit kernel) that plans without a
-tiling of their own take for bin- and quad-major frames: equal to the oracle,
+tiling of their own take, in all three layouts: equal to the oracle,
 and to the fused look-back kernel (a plan with a tiling), word for word, at
 the edges of its tiles (rows per band 8, 16 and 32, superbands of 4 bands, 64
-and 128 columns, segments of 8 chunks), for every binning, pitched and
+and 128 columns, segments of 8 chunks, 32 and 64 bins of a pixel's record), for every binning, pitched and
 unaligned frames and unaligned outputs.  Counts are integers: no tolerance."""
 import numpy as np
 import pytest
@@ -34,6 +34,8 @@ def laid_out(ref, layout):
     if layout == ihist.IHIST_QUAD_MAJOR:
         b, h, w = ref.shape
         return np.ascontiguousarray(ref.reshape(b // 4, 4, h, w).transpose(0, 2, 3, 1))
+    if layout == ihist.IHIST_PIXEL_MAJOR:
+        return np.ascontiguousarray(ref.transpose(1, 2, 0))
     return ref
 
 
@@ -59,11 +61,11 @@ def computed(plan, frame, shift=0):
     return u32(out).reshape(plan.out_shape)
 
 
-@pytest.mark.parametrize("layout", [ihist.IHIST_BIN_MAJOR, ihist.IHIST_QUAD_MAJOR])
+@pytest.mark.parametrize("layout", [ihist.IHIST_BIN_MAJOR, ihist.IHIST_QUAD_MAJOR, ihist.IHIST_PIXEL_MAJOR])
 @pytest.mark.parametrize("h,w,nbins", [
     (1, 1, 1), (7, 63, 4), (8, 64, 5), (9, 65, 12), (31, 127, 256), (32, 128, 253), (33, 129, 8), (65, 1023, 3),
     (64, 1024, 16), (127, 1025, 24), (129, 2049, 4), (257, 260, 64), (600, 640, 32), (2049, 130, 8), (2, 6000, 4),
-    (140, 1921, 100)])
+    (140, 1921, 100), (40, 200, 72), (70, 161, 33)])
 def test_edges_of_the_tiles(h, w, nbins, layout):
     if layout == ihist.IHIST_QUAD_MAJOR:
         nbins = (nbins + 3) // 4 * 4
@@ -75,7 +77,7 @@ def test_edges_of_the_tiles(h, w, nbins, layout):
         assert np.array_equal(got, ref), (pad, offset, shift)
 
 
-@pytest.mark.parametrize("layout", [ihist.IHIST_BIN_MAJOR, ihist.IHIST_QUAD_MAJOR])
+@pytest.mark.parametrize("layout", [ihist.IHIST_BIN_MAJOR, ihist.IHIST_QUAD_MAJOR, ihist.IHIST_PIXEL_MAJOR])
 @pytest.mark.parametrize("h,w", [(33, 200), (300, 1100)])
 @pytest.mark.parametrize("nbins", [4, 252, 256])
 def test_tables_with_values_in_no_bin(h, w, nbins, layout):
@@ -95,7 +97,7 @@ def test_joint_bins(bins):
             assert np.array_equal(computed(plan, on_gpu(img, 7, 1)), ref)
 
 
-@pytest.mark.parametrize("layout", [ihist.IHIST_BIN_MAJOR, ihist.IHIST_QUAD_MAJOR])
+@pytest.mark.parametrize("layout", [ihist.IHIST_BIN_MAJOR, ihist.IHIST_QUAD_MAJOR, ihist.IHIST_PIXEL_MAJOR])
 @pytest.mark.parametrize("h,w,nbins", [(1080, 1920, 64), (1081, 1921, 20), (2100, 3000, 12), (240, 320, 16),
                                        (61, 40000, 8), (8192, 700, 8)])
 @pytest.mark.parametrize("overlap", [0, 1])
