@@ -53,7 +53,8 @@ struct BandDesc {
   int H, W, B, qmul;
   int early;            // 1: the frame may be read before the previous grid has completed
   int R, nbands, nsb, nq, nchunks, nsegs, cps;
-  int split;  // a count thread counts R >> split pixels
+  int split;     // a count thread counts R >> split pixels
+  int wpg, gpc;  // emit CTAs: warps of one group, and groups
   uint8_t *q;
   int bpb, nblk;  // pixel-major: bins of one CTA (a multiple of 4, at most 64) and blocks of them
   uint32_t *pb, *sb, *rl, *rls;
@@ -172,10 +173,8 @@ __host__ __device__ inline size_t count_smem_bytes(const BandDesc &f) {
 // columns' and rows' counts.  Grid: x over half chunks, y over column tiles
 // of rows; z = 0 column tiles, 1 row tiles (two per column tile).
 template <int MODE>
-__global__ void __launch_bounds__(kCountThreads, 4) band_count_kernel(const __grid_constant__ BandDesc f) {
-  extern __shared__ __align__(16) uint8_t smem_raw[];
+__device__ __forceinline__ void band_count(const BandDesc &f, uint8_t *smem_raw, const uint3 block) {
   __shared__ uint8_t s_lut[MODE == kBinTable ? 256 : 1];
-  if (!f.early) griddep_wait();
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   uint32_t *tile32 = reinterpret_cast<uint32_t *>(smem_raw);
   uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + count_tile_bytes(f));
@@ -184,7 +183,7 @@ __global__ void __launch_bounds__(kCountThreads, 4) band_count_kernel(const __gr
   if constexpr (MODE == kBinTable) {
     const uint32_t none = 4u * (uint32_t)f.nq;  // counted in the extra word, matched by no group
     if (t < 256) {
-      const uint32_t e = __ldg(f.lut + t);
+      const uint32_t e = __ldcg(f.lut + t);
       s_lut[t] = (uint8_t)((e >> 3) < (uint32_t)f.B ? e >> 3 : none);
     }
     __syncthreads();
@@ -195,9 +194,9 @@ __global__ void __launch_bounds__(kCountThreads, 4) band_count_kernel(const __gr
     for (int e = t; e < (f.nq + 1) * (kCountThreads / 4); e += kCountThreads)
       reinterpret_cast<uint4 *>(hist)[e] = make_uint4(0u, 0u, 0u, 0u);
   };
-  if (blockIdx.z == 0) {
-    const int hc = blockIdx.x;
-    const int y0 = blockIdx.y * col_tile_rows(f), nrows = min(col_tile_rows(f), f.H - y0);
+  if (block.z == 0) {
+    const int hc = block.x;
+    const int y0 = block.y * col_tile_rows(f), nrows = min(col_tile_rows(f), f.H - y0);
     const int x4 = hc * kHalf + 4 * (t & 15);
     const int tcol = (t >> 4) * (kColPitch / 4) + (t & 15);
     constexpr int kRowStep = kCountThreads / 16, kTileStep = kRowStep * (kColPitch / 4);
@@ -228,7 +227,7 @@ __global__ void __launch_bounds__(kCountThreads, 4) band_count_kernel(const __gr
     __syncthreads();
     // thread (column, every eighth group): down each superband's bands
     const size_t band_step = (size_t)f.nq * wpad;
-    const int sb0 = blockIdx.y << 1 >> f.split, sb1 = min(sb0 + (2 >> f.split), f.nsb);
+    const int sb0 = block.y << 1 >> f.split, sb1 = min(sb0 + (2 >> f.split), f.nsb);
     for (int g = piece; g < f.nq; g += kCountThreads / kHalf) {
       const uint32_t *hg = hist + g * kCountThreads + x;
       const size_t at = (size_t)g * wpad + hc * kHalf + x;
@@ -252,9 +251,9 @@ __global__ void __launch_bounds__(kCountThreads, 4) band_count_kernel(const __gr
       }
     }
   } else {
-    const int c = blockIdx.x >> 1;
+    const int c = block.x >> 1;
     const int trows = row_tile_rows(f), lr = __ffs(trows) - 1;
-    const int y0 = (2 * blockIdx.y + (blockIdx.x & 1)) * trows, nrows = min(trows, f.H - y0);
+    const int y0 = (2 * block.y + (block.x & 1)) * trows, nrows = min(trows, f.H - y0);
     load_tile<MODE>(f, s_lut, y0, w, kCountThreads / 32, nrows, c * kChunk + 4 * lane,
                     tile32 + w * (kRowPitch / 4) + lane, kCountThreads / 32 * (kRowPitch / 4), false);
     clear();
@@ -320,8 +319,65 @@ __global__ void __launch_bounds__(kCountThreads, 4) band_count_kernel(const __gr
       }
     }
   }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kCountThreads, 4) band_count_kernel(const __grid_constant__ BandDesc f) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  if (!f.early) griddep_wait();
+  band_count<MODE>(f, smem_raw, blockIdx);
   griddep_release();
 }
+
+// CTAs of one frame, in the order (z, y, x) of the grid above.
+__host__ __device__ inline unsigned int count_ctas(const BandDesc &f) {
+  return 4u * (unsigned)f.nchunks * (unsigned)((f.H + col_tile_rows(f) - 1) / col_tile_rows(f));
+}
+
+// Batches: the frames of one launch, as the running count of their CTAs.
+// (By value: the search reads the constant bank.  A batch of more frames
+// takes several launches.)
+constexpr int kBatchFrames = 256;
+struct BandBatch {
+  const BandDesc *frames;
+  int n;
+  unsigned int end[kBatchFrames];
+};
+
+// This CTA's frame, copied to shared memory (with loads that see what the
+// copy before this launch wrote), and its index among the frame's CTAs.
+__device__ __forceinline__ unsigned int batch_frame(const BandBatch &b, BandDesc *s_desc) {
+  int lo = 0, hi = b.n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (b.end[mid] > blockIdx.x) hi = mid; else lo = mid + 1;
+  }
+  constexpr int kWords = (int)(sizeof(BandDesc) / 4);
+  static_assert(sizeof(BandDesc) % 4 == 0 && kWords <= 128, "one word per thread");
+  if (threadIdx.x < kWords)
+    reinterpret_cast<uint32_t *>(s_desc)[threadIdx.x] =
+        ld_relaxed_u32(reinterpret_cast<const uint32_t *>(b.frames + lo) + threadIdx.x);
+  __syncthreads();
+  return blockIdx.x - (lo > 0 ? b.end[lo - 1] : 0u);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kCountThreads, 4) band_count_batch_kernel(const __grid_constant__ BandBatch b) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  __shared__ BandDesc s_desc;
+  griddep_wait();
+  unsigned int it = batch_frame(b, &s_desc);
+  const BandDesc &f = s_desc;
+  uint3 block;
+  block.x = it % (2u * f.nchunks);
+  it /= 2u * f.nchunks;
+  const unsigned int ny = (unsigned)(f.H + col_tile_rows(f) - 1) / (unsigned)col_tile_rows(f);
+  block.y = it % ny;
+  block.z = it / ny;
+  band_count<MODE>(f, smem_raw, block);
+  griddep_release();
+}
+
 
 // Inclusive prefix of v[0..3] (this lane's 4 columns) over the chunk.
 __device__ __forceinline__ void chunk_prefix(uint32_t v[4], int lane) {
@@ -351,8 +407,14 @@ __host__ __device__ inline size_t emit_smem_bytes(int warps, int R) { return (si
 // after the scan the lanes exchange columns through shared memory, from 4
 // neighbouring ones per lane to columns lane, lane + 32, .. -- one word per
 // column for the four bins, so the exchange costs 5 accesses a row.
+//
+// planes: items run through the bands of one group before the next, so that
+// the CTAs of many frames write few planes at a time (64 frames of 1920x1080
+// x 64, bin-major: 5.71 -> 5.65 ms with their queries; quad-major, whose rows
+// are four times as long, 2.55 -> 2.59 for 32 frames, so it keeps the band
+// order, in which a single frame is as fast).
 template <int LAYOUT, bool VEC>
-__global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4) band_emit_kernel(const __grid_constant__ BandDesc f) {
+__device__ __forceinline__ void band_emit(const BandDesc &f, uint8_t *smem_raw, unsigned int it, bool planes) {
   __shared__ uint4 s_row[kSegWarps][32];   // per chunk: counts left of it, per row of the band
   __shared__ uint2 s_own[kSegWarps][32];   // per chunk: its own counts, per row (16-bit lanes)
   __shared__ uint2 s_left[kSegWarps][32];  // per warp: its share of the chunks left of the segment
@@ -361,18 +423,17 @@ __global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4) b
   constexpr bool SPREAD = LAYOUT == 0 && !VEC;
   constexpr int P = 4;  // rows in hand at a time
   __shared__ __align__(16) uint32_t s_col[SPREAD ? kSegWarps : 1][SPREAD ? 4 : 1][SPREAD ? kChunk : 4];
-  extern __shared__ __align__(16) uint8_t smem_raw[];  // per chunk: the band's bins, R rows of 128 bytes
-  griddep_wait();
-  griddep_release();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  unsigned int it = blockIdx.x;
   const int seg = (int)(it % (unsigned)f.nsegs);
   it /= (unsigned)f.nsegs;
-  const int g = (int)(it % (unsigned)f.nq);
-  const int k = (int)(it / (unsigned)f.nq);
+  const unsigned int ngs = (unsigned)(f.nq + f.gpc - 1) / (unsigned)f.gpc;
+  const int lg = w / f.wpg, w0 = lg * f.wpg;  // this warp's group in the CTA, and that group's first warp
+  const int gs = (int)(planes ? it / (unsigned)f.nbands : it % ngs) * f.gpc;
+  const int g = gs + lg;
+  const int k = (int)(planes ? it % (unsigned)f.nbands : it / ngs);
   const int c0 = seg * f.cps;
-  const int c = c0 + w;
-  const bool live = c < f.nchunks;
+  const int c = c0 + w - w0;
+  const bool live = lg < f.gpc && g < f.nq && c < f.nchunks;
   const int y0 = k * f.R;
   const int nrows = min(f.R, f.H - y0);
   const size_t wpad = (size_t)f.nchunks * kChunk;
@@ -420,10 +481,11 @@ __global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4) b
     s_own[w][lane] = o;
   }
   if (seg > 0) {
-    // the chunks left of the segment, shared out over the CTA's warps
+    // the chunks left of the segment, shared out over the CTA's warps (which
+    // hold one group then)
     uint2 l = make_uint2(0u, 0u);
     for (int cl = w; cl < c0; cl += nw)
-      if (lane < f.R) add_bytes16(l.x, l.y, __ldcg(f.rl + ((size_t)cl * f.nq + g) * hpad + y0 + lane));
+      if (lane < f.R) add_bytes16(l.x, l.y, __ldcg(f.rl + ((size_t)cl * f.nq + gs) * hpad + y0 + lane));
     s_left[w][lane] = l;
     uint4 tot = make_uint4(0u, 0u, 0u, 0u);
     auto add = [&](uint2 v) {
@@ -434,7 +496,7 @@ __global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4) b
     };
 #pragma unroll 4
     for (int cl = w; cl < c0; cl += nw)
-      for (int j = lane; j < k; j += 32) add(__ldcg(f.ct + ((size_t)g * f.nchunks + cl) * f.nbands + j));
+      for (int j = lane; j < k; j += 32) add(__ldcg(f.ct + ((size_t)gs * f.nchunks + cl) * f.nbands + j));
     tot.x = __reduce_add_sync(kFull, tot.x);
     tot.y = __reduce_add_sync(kFull, tot.y);
     tot.z = __reduce_add_sync(kFull, tot.z);
@@ -447,7 +509,7 @@ __global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4) b
   {
     uint4 l = make_uint4(0u, 0u, 0u, 0u);
     uint2 r = make_uint2(0u, 0u);
-    for (int i = 0; i < w; ++i) {
+    for (int i = w0; i < w; ++i) {
       const uint4 v = s_tot[i];
       l.x += v.x; l.y += v.y; l.z += v.z; l.w += v.w;
       const uint2 o = s_own[i][lane];
@@ -587,6 +649,27 @@ __global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4) b
   }
 }
 
+template <int LAYOUT, bool VEC>
+__global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4)
+    band_emit_kernel(const __grid_constant__ BandDesc f) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];  // per chunk: the band's bins, R rows of 128 bytes
+  griddep_wait();
+  griddep_release();
+  band_emit<LAYOUT, VEC>(f, smem_raw, blockIdx.x, false);
+}
+
+template <int LAYOUT, bool VEC>
+__global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4)
+    band_emit_batch_kernel(const __grid_constant__ BandBatch b) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  __shared__ BandDesc s_desc;
+  griddep_wait();
+  griddep_release();
+  const unsigned int it = batch_frame(b, &s_desc);
+  const BandDesc f = s_desc;
+  band_emit<LAYOUT, VEC>(f, smem_raw, it, LAYOUT == 0);
+}
+
 // Pixel-major H[y][x][b].  One CTA per (band, block of bins, chunk), one warp
 // per 32 columns of the chunk and 32 * NJ bins of the block; a lane holds NJ
 // bins (32 apart) of all 32 columns, so that a pixel's counts leave as
@@ -638,18 +721,14 @@ __device__ __forceinline__ void emit_strip(const BandDesc &f, uint32_t (&acc)[kS
 }
 
 template <int WARPS, int NJ>
-__global__ void __launch_bounds__(WARPS * 32, NJ == 2 ? 4 : 24 / WARPS) band_emit_pixel_kernel(const __grid_constant__ BandDesc f) {
-  extern __shared__ __align__(16) uint8_t smem_raw[];
+__device__ __forceinline__ void band_emit_pixel(const BandDesc &f, uint8_t *smem_raw, unsigned int it) {
   // first rows of H [column][16-byte unit of 4 bins ^ (column / 4 mod 8)], then
   // the counts left of each strip [strip][row][8-byte unit of 4 bins ^ (row
   // mod 16)], then the band's bins [row][column]
   uint4 *s_top = reinterpret_cast<uint4 *>(smem_raw);
   uint2 *s_left = reinterpret_cast<uint2 *>(smem_raw + kPixelTopBytes);
   constexpr int kUnits = kPixelBins / 4;
-  griddep_wait();
-  griddep_release();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  unsigned int it = blockIdx.x;
   const int c = (int)(it % (unsigned)f.nchunks);
   it /= (unsigned)f.nchunks;
   const int blk = (int)(it % (unsigned)f.nblk);
@@ -751,6 +830,27 @@ __global__ void __launch_bounds__(WARPS * 32, NJ == 2 ? 4 : 24 / WARPS) band_emi
     emit_strip<NJ, true>(f, acc, bin, has, left, tile + kStripCols * strip, y0, nrows, x0, ncols, b0);
   else
     emit_strip<NJ, false>(f, acc, bin, has, left, tile + kStripCols * strip, y0, nrows, x0, ncols, b0);
+}
+
+template <int WARPS, int NJ>
+__global__ void __launch_bounds__(WARPS * 32, NJ == 2 ? 4 : 24 / WARPS)
+    band_emit_pixel_kernel(const __grid_constant__ BandDesc f) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  griddep_wait();
+  griddep_release();
+  band_emit_pixel<WARPS, NJ>(f, smem_raw, blockIdx.x);
+}
+
+template <int WARPS, int NJ>
+__global__ void __launch_bounds__(WARPS * 32, NJ == 2 ? 4 : 24 / WARPS)
+    band_emit_pixel_batch_kernel(const __grid_constant__ BandBatch b) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  __shared__ BandDesc s_desc;
+  griddep_wait();
+  griddep_release();
+  const unsigned int it = batch_frame(b, &s_desc);
+  const BandDesc f = s_desc;
+  band_emit_pixel<WARPS, NJ>(f, smem_raw, it);
 }
 
 }  // namespace ihist

@@ -1,5 +1,6 @@
 // ihist_bands_host.h -- host interface of the two-launch path
-// (ihist_bands.cu), used by plans (ihist_api.cu).
+// (ihist_bands.cu), used by plans (ihist_api.cu) and batches
+// (ihist_batch_api.cu).
 #pragma once
 
 #include "ihist_bands.cuh"
@@ -8,19 +9,46 @@
 namespace ihist {
 namespace host {
 
-// Whether a frame takes the two-launch path, and its shape fields in *f.
+// Emit kernels: 0, 1 bin-major (rows 16-byte aligned or not), 2, 3 quad-major
+// (likewise), 4, 5, 6 pixel-major (at most 32 bins a block, one bin per lane,
+// two bins per lane).
+constexpr int kBandKinds = 7;
+inline int bands_kind_layout(int kind) {
+  return kind < 2 ? IHIST_BIN_MAJOR : kind < 4 ? IHIST_QUAD_MAJOR : IHIST_PIXEL_MAJOR;
+}
+int bands_kind(const BandDesc &f, int layout);
+unsigned int bands_threads(const BandDesc &f, int kind);
+
+// Whether the two-launch path is the faster one for a frame of this size.
+bool bands_fit(int h, int w, int layout);
+
+// The shape fields of a frame with R rows per band.
+void bands_describe(int h, int w, int nbins, int layout, int R, int split, BandDesc *f);
+
+// Whether a plan's frames take the two-launch path, and their shape in *f.
 bool bands_shape(int h, int w, int nbins, int layout, int sms, BandDesc *f);
 
 // Workspace bytes of the shape; with a base (256-byte aligned), also the
-// pointers into it.
-size_t bands_layout(BandDesc *f, char *base);
+// pointers into it.  any_layout: enough for the same shape in every layout.
+size_t bands_layout(BandDesc *f, char *base, bool any_layout = false);
 
-// Let the kernels of this binning and layout use their shared memory (optin: the
-// largest a CTA may have).
+// Let the kernels of this binning and layout (or all batch kernels) use the
+// shared memory they need (optin: the largest a CTA may have).
 int bands_prepare(const BandDesc &f, int mode, int layout, size_t optin);
+int bands_prepare_batch(size_t optin);
 
-// Both launches, with programmatic stream serialization.
+// Both launches of one frame, with programmatic stream serialization.
 int launch_bands(const BandDesc &f, int mode, int layout, void *stream);
+
+// One launch of a batch: n frames (at most kBatchFrames) through the count
+// kernel of a binning or the emit kernel of a kind; their descriptors on the
+// device and on the host.
+struct BandRun {
+  bool count;
+  int kernel, n;
+  const BandDesc *d_desc, *h_desc;
+};
+int launch_bands_batch(const BandRun *runs, int nruns, void *stream);
 
 }  // namespace host
 }  // namespace ihist

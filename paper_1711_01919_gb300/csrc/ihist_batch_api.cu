@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "ihist.h"
+#include "ihist_bands_host.h"
 #include "ihist_host.h"
 #include "ihist_kernels.h"
 #include "ihist_query.cuh"
@@ -201,6 +202,15 @@ struct ihist_batch_s {
   std::vector<uint8_t *> slot_idx;
   std::vector<FrameDesc> fd;                          // current frames
   std::vector<ihist_frame_t> io;
+  // The two-launch path (ihist_bands.cuh): a slot's band workspace shares the
+  // memory of its look-back carries, since a launch goes one way or the other.
+  bool band_ok;                        // the batch was planned without a tiling
+  int band_R, band_split;
+  std::vector<char *> slot_base;
+  std::vector<size_t> slot_bytes;
+  BandDesc *d_bc, *d_be;               // descriptors by count kernel and by emit kernel
+  std::vector<BandDesc> bc, be;        // the current binding's, in those orders
+  std::vector<BandRun> runs;           // its launches; empty: the look-back kernel
   // Pinned staging of the descriptors, two sets used by alternate bindings:
   // a binding waits only for the copy made from its set two bindings ago,
   // so a caller can bind and launch ahead of the GPU.  h_* point at the set
@@ -210,6 +220,7 @@ struct ihist_batch_s {
     CUtensorMap *tm;
     unsigned int *end, *bins_end;
     uint32_t *lut;
+    BandDesc *bc, *be;
   } stage_sets[2];
   cudaEvent_t staged[2];
   int stage_cur;
@@ -232,6 +243,81 @@ static bool encode_frame_map(const uint8_t *in, size_t pitch, int h, int w, int 
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t *>(in), gdim, gstride,
              box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Describe the frames for the two-launch path, in launch order; false if one
+// of them does not take it or does not fit its slot.
+static bool bands_bind(ihist_batch_s *b, const ihist_frame_t *frames, const std::vector<FrameDesc> &fd, int n,
+                       std::vector<BandDesc> *bc, std::vector<BandDesc> *be, std::vector<BandRun> *runs) {
+  if (!b->band_ok) return false;
+  // Large bin-major batches with aligned rows hide the look-back kernel's
+  // chain behind their stores: 8, 16 and 64 frames of 1920x1080 x 64 take
+  // 666, 1316 and 5227 us here against 722, 1365 and 5210 there.  Other
+  // layouts and odd widths store better here at any size (32 quad-major
+  // frames 2549 against 2791 us, 8 pixel-major 708 / 1051, 8 of 1921x1080
+  // 735 / 1680).
+  size_t plain = 0;
+  bool other = false;
+  for (int i = 0; i < n; ++i) {
+    plain += ihist_output_bytes(frames[i].h, frames[i].w, frames[i].nbins);
+    other = other || frames[i].layout != IHIST_BIN_MAJOR || !frame_vec_ok(frames[i]);
+  }
+  if (!other && plain > (16ull << 30)) return false;
+  std::vector<BandDesc> desc(n);
+  std::vector<int> mode(n), kind(n), order(n);
+  for (int i = 0; i < n; ++i) {
+    const ihist_frame_t &fr = frames[i];
+    if (!bands_fit(fr.h, fr.w, fr.layout)) return false;
+    BandDesc &f = desc[i];
+    bands_describe(fr.h, fr.w, fr.nbins, fr.layout, b->band_R, b->band_split, &f);
+    if (!f.nblk && f.nsegs == 1) f.gpc = std::max(1, std::min(f.nq, kSegWarps / f.wpg));
+    if (bands_layout(&f, b->slot_base[i]) > b->slot_bytes[i]) return false;
+    f.in = fr.d_in;
+    f.pitch = (long long)fr.in_pitch;
+    f.out = fr.d_out;
+    f.ctrl = b->ctrl;
+    mode[i] = kBinUniform;
+    if (fr.bin_of_value) {
+      mode[i] = kBinTable;
+      f.lut = fd[i].lut;
+      if (fr.nbins > 252)  // no byte left for "no bin"
+        for (int v = 0; v < 256; ++v)
+          if (fr.bin_of_value[v] < 0) return false;
+    } else if (frame_joint(fr)) {
+      mode[i] = kBinJoint;
+      f.jc = fr.channels;
+      int stride = 1;
+      for (int c = fr.channels - 1; c >= 0; --c) {
+        f.jmul[c] = fr.bins_per_channel[c];
+        f.jstride[c] = stride;
+        stride *= f.jmul[c];
+      }
+    }
+    kind[i] = bands_kind(f, fr.layout);
+    order[i] = i;
+  }
+  bc->clear();
+  be->clear();
+  runs->clear();
+  for (int pass = 0; pass < 2; ++pass) {
+    const std::vector<int> &key = pass ? kind : mode;
+    std::vector<BandDesc> *to = pass ? be : bc;
+    // by kernel, then largest first, so that a launch ends on small frames
+    std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
+      if (key[a] != key[c]) return key[a] < key[c];
+      return ihist_output_bytes(frames[a].h, frames[a].w, frames[a].nbins) >
+             ihist_output_bytes(frames[c].h, frames[c].w, frames[c].nbins);
+    });
+    for (int i = 0; i < n; ++i) {
+      to->push_back(desc[order[i]]);
+      const int kernel = key[order[i]];
+      if (i == 0 || runs->back().count != (pass == 0) || runs->back().kernel != kernel ||
+          runs->back().n == kBatchFrames)
+        runs->push_back(BandRun{pass == 0, kernel, 0, (pass ? b->d_be : b->d_bc) + i, nullptr});
+      ++runs->back().n;
+    }
+  }
+  return true;
 }
 
 // Point h_* at staging set i.
@@ -320,6 +406,18 @@ static int batch_bind(ihist_batch_s *b, const ihist_frame_t *frames, int n) {
     b->h_end[k] = (unsigned int)run;
     b->h_fd[k] = fd[i];
   }
+  std::vector<BandDesc> bc, be;
+  std::vector<BandRun> runs;
+  if (bands_bind(b, frames, fd, n, &bc, &be, &runs)) {
+    std::memcpy(b->stage_sets[b->stage_cur].bc, bc.data(), (size_t)n * sizeof(BandDesc));
+    std::memcpy(b->stage_sets[b->stage_cur].be, be.data(), (size_t)n * sizeof(BandDesc));
+  } else {
+    runs.clear();
+  }
+  b->bc.swap(bc);
+  b->be.swap(be);
+  b->runs.swap(runs);
+  for (BandRun &r : b->runs) r.h_desc = r.count ? b->bc.data() + (r.d_desc - b->d_bc) : b->be.data() + (r.d_desc - b->d_be);
   b->fd.assign(fd.begin(), fd.end());
   b->io.assign(frames, frames + n);
   b->n = n;
@@ -340,6 +438,11 @@ static int batch_upload(ihist_batch_s *b, cudaStream_t s) {
           cudaSuccess ||
       (b->lut && cudaMemcpyAsync(b->d_lut, b->h_lut, (size_t)n * 256 * sizeof(uint32_t), cudaMemcpyHostToDevice,
                                  s) != cudaSuccess) ||
+      (!b->runs.empty() &&
+       (cudaMemcpyAsync(b->d_bc, b->stage_sets[b->stage_cur].bc, (size_t)n * sizeof(BandDesc), cudaMemcpyHostToDevice,
+                        s) != cudaSuccess ||
+        cudaMemcpyAsync(b->d_be, b->stage_sets[b->stage_cur].be, (size_t)n * sizeof(BandDesc), cudaMemcpyHostToDevice,
+                        s) != cudaSuccess)) ||
       cudaEventRecord(b->staged[b->stage_cur], s) != cudaSuccess)
     return IHIST_ERR_CUDA;
   return IHIST_OK;
@@ -364,6 +467,8 @@ extern "C" void ihist_batch_destroy(ihist_batch_t b) {
     if (st.end) cudaFreeHost(st.end);
     if (st.bins_end) cudaFreeHost(st.bins_end);
     if (st.lut) cudaFreeHost(st.lut);
+    if (st.bc) cudaFreeHost(st.bc);
+    if (st.be) cudaFreeHost(st.be);
   }
   if (b->ws) cudaFree(b->ws);
   if (prev != b->device && prev >= 0) cudaSetDevice(prev);
@@ -376,6 +481,9 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
   ihist_tune_t t;
   std::memset(&t, 0, sizeof(t));
   if (tune) t = *tune;
+  // the two-launch path takes batches with no tiling of their own
+  const bool tiled = t.rows_per_band || t.bins_per_cta || t.warps_per_cta || t.ctas_per_sm || t.chunks_per_warp ||
+                     t.groups_per_cta || t.fault_skip_band >= 1;
   // frames with value -> bin tables make a table batch (every frame bins
   // through a table; 4 or 8 bins per CTA)
   bool lut = false;
@@ -538,6 +646,36 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
       b->ctas_per_sm[tma][vec] = t.ctas_per_sm > 0 ? std::min(t.ctas_per_sm, occ) : occ;
     }
 
+  // The two-launch path: one band height for all frames, by the rules of
+  // single frames on their sum, and room for each frame's counts.
+  b->band_ok = !tiled && bands_prepare_batch((size_t)optin) == IHIST_OK;
+  std::vector<size_t> band_bytes(n, 0);
+  if (b->band_ok) {
+    auto sum = [&](int R, bool pixel) {
+      long long v = 0;
+      for (int i = 0; i < n; ++i) {
+        BandDesc f;
+        if ((frames[i].layout == IHIST_PIXEL_MAJOR) != pixel) continue;
+        bands_describe(frames[i].h, frames[i].w, frames[i].nbins, frames[i].layout, R, 0, &f);
+        v += (long long)f.nbands * f.nchunks * (pixel ? f.nblk : f.nq);
+      }
+      return v;
+    };
+    int h_max = 0;
+    for (int i = 0; i < n; ++i) h_max = std::max(h_max, frames[i].h);
+    b->band_R = sum(32, false) >= 16000 || sum(32, true) >= 400 || h_max > 2048 ? 32
+                : sum(16, false) >= 600 || sum(16, true) >= 120                 ? 16
+                                                                                : 8;
+    unsigned long long ctas = 0;
+    for (int i = 0; i < n; ++i) {
+      BandDesc f;
+      bands_describe(frames[i].h, frames[i].w, frames[i].nbins, frames[i].layout, b->band_R, 0, &f);
+      ctas += count_ctas(f);
+      if (bands_fit(frames[i].h, frames[i].w, frames[i].layout)) band_bytes[i] = bands_layout(&f, nullptr, true);
+    }
+    b->band_split = ctas < 2ull * sms ? 1 : 0;
+  }
+
   // workspace: control block and flags (cleared), descriptor arrays
   // (written only by copies), then each slot's carries
   size_t off = 0;
@@ -552,6 +690,10 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
   off = align_up(off + (size_t)n * sizeof(FrameDesc), 256);
   const size_t o_tm = off;
   off = align_up(off + (size_t)n * sizeof(CUtensorMap), 256);
+  const size_t o_bc = off;
+  off = align_up(off + (size_t)n * sizeof(BandDesc), 256);
+  const size_t o_be = off;
+  off = align_up(off + (size_t)n * sizeof(BandDesc), 256);
   const size_t o_end = off;
   off = align_up(off + (size_t)n * sizeof(unsigned int), 256);
   const size_t o_bend = off;
@@ -561,10 +703,13 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
   const size_t o_carry = off;
   for (int i = 0; i < n; ++i) {
     const size_t nci = b->slot_nci[i];
+    const size_t at = off;
     off = align_up(off + nci * kChunk * (b->G / 4) * 4, 256);
     off = align_up(off + nci * b->G * 4, 256);
     off = align_up(off + nci * b->G * kChunk * 4, 256);
     off = align_up(off + b->slot_hwords[i] * 4, 256);
+    off = std::max(off, at + band_bytes[i]);
+    b->slot_bytes.push_back(off - at);
   }
   const size_t o_idx = off;  // joint-bin planes of the slots planned with joint frames
   for (int i = 0; i < n; ++i) {
@@ -582,6 +727,8 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
               cudaMallocHost((void **)&st.end, (size_t)n * sizeof(unsigned int)) != cudaSuccess ||
               cudaMallocHost((void **)&st.bins_end, (size_t)n * sizeof(unsigned int)) != cudaSuccess ||
               (lut && cudaMallocHost((void **)&st.lut, (size_t)n * 256 * sizeof(uint32_t)) != cudaSuccess) ||
+              cudaMallocHost((void **)&st.bc, (size_t)n * sizeof(BandDesc)) != cudaSuccess ||
+              cudaMallocHost((void **)&st.be, (size_t)n * sizeof(BandDesc)) != cudaSuccess ||
               cudaEventCreateWithFlags(&b->staged[i], cudaEventDisableTiming) != cudaSuccess)
             return false;
         }
@@ -598,6 +745,8 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
   b->d_fd = reinterpret_cast<FrameDesc *>(base + o_fd);
   b->d_fdq = reinterpret_cast<FrameDesc *>(base + o_fdq);
   b->d_tm = reinterpret_cast<CUtensorMap *>(base + o_tm);
+  b->d_bc = reinterpret_cast<BandDesc *>(base + o_bc);
+  b->d_be = reinterpret_cast<BandDesc *>(base + o_be);
   b->d_end = reinterpret_cast<unsigned int *>(base + o_end);
   b->d_bins_end = reinterpret_cast<unsigned int *>(base + o_bend);
   if (lut) b->d_lut = reinterpret_cast<uint32_t *>(base + o_lut);
@@ -608,6 +757,8 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
     fo += nci * sizeof(uint32_t);
     b->slot_hflags.push_back(reinterpret_cast<uint32_t *>(base + fo));  // segment flags, cleared with the rest
     fo += b->slot_nhs[i] * sizeof(uint32_t);
+    b->slot_base.push_back(base + co);
+    const size_t next = co + b->slot_bytes[i];
     b->slot_cnt.push_back(reinterpret_cast<uint32_t *>(base + co));
     co = align_up(co + nci * kChunk * (b->G / 4) * 4, 256);
     b->slot_left.push_back(reinterpret_cast<uint32_t *>(base + co));
@@ -615,7 +766,7 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
     b->slot_incl.push_back(reinterpret_cast<uint32_t *>(base + co));
     co = align_up(co + nci * b->G * kChunk * 4, 256);
     b->slot_hagg.push_back(reinterpret_cast<uint32_t *>(base + co));
-    co = align_up(co + b->slot_hwords[i] * 4, 256);
+    co = next;
   }
   size_t xo = o_idx;
   for (int i = 0; i < n; ++i) {
@@ -679,10 +830,29 @@ extern "C" int ihist_batch_set_io(ihist_batch_t b, const ihist_frame_t *frames, 
   return batch_upload(b, (cudaStream_t)stream);
 }
 
+// A captured launch has to follow later bindings when it is replayed.  The
+// look-back launch reads its work-list on the device; the two-launch path's
+// grids are those of the binding at the call, so it is not captured.
+static bool under_capture(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
 extern "C" int ihist_batch_compute(ihist_batch_t b, void *stream) {
   if (!b) return IHIST_ERR_INVALID_ARG;
   int rc = check_batch_device(b);
   if (rc != IHIST_OK) return rc;
+  if (!b->runs.empty() && !under_capture((cudaStream_t)stream)) {
+    rc = launch_bands_batch(b->runs.data(), (int)b->runs.size(), stream);
+    if (rc != IHIST_OK) return rc;
+    if (cudaEventRecord(b->computed, (cudaStream_t)stream) != cudaSuccess) return IHIST_ERR_CUDA;
+    b->launched = true;
+    return IHIST_OK;
+  }
   // joint frames: their joint-bin planes first (the scan waits for them)
   for (int i = 0; i < b->n; ++i) {
     const ihist_frame_t &fr = b->io[i];
