@@ -52,10 +52,12 @@ __global__ void __launch_bounds__(256) query_kernel(const uint32_t *__restrict__
                : LAYOUT == 1 ? ((size_t)y * W + x) * (size_t)B + b
                              : ((size_t)(b >> 2) * plane + (size_t)y * W + x) * 4 + (b & 3);
       };
-      v = __ldg(hist + at(y1, x1));
-      if (y0 > 0) v -= __ldg(hist + at(y0 - 1, x1));
-      if (x0 > 0) v -= __ldg(hist + at(y1, x0 - 1));
-      if (x0 > 0 && y0 > 0) v += __ldg(hist + at(y0 - 1, x0 - 1));
+      // all four loads before the first use, so that they are in flight together
+      const uint32_t br = __ldg(hist + at(y1, x1));
+      const uint32_t tr = y0 > 0 ? __ldg(hist + at(y0 - 1, x1)) : 0u;
+      const uint32_t bl = x0 > 0 ? __ldg(hist + at(y1, x0 - 1)) : 0u;
+      const uint32_t tl = x0 > 0 && y0 > 0 ? __ldg(hist + at(y0 - 1, x0 - 1)) : 0u;
+      v = br - tr - bl + tl;
     } else if (b == 0) {
       latch_status(ctrl, kStatusBadRect);
     }
