@@ -90,6 +90,8 @@ _lib = None
 def load(path: str = LIB_PATH):
     """Load libihist.so and declare its signatures (once)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -433,10 +435,20 @@ def ihist_batch_destroy(batch: int) -> None:
 
 # --------------------------------------------------------------- torch glue
 
-def _stream(stream):
+def _current_raw_stream():
+    """The current stream's handle.  torch.cuda.current_stream() builds a
+    Stream object on the way (3.0 us of a 640x480 frame's 16.6 us of host
+    time per call, compute and query each); the raw lookup takes 0.3 us."""
     import torch
-    if stream is None:
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None or not torch.cuda.is_initialized():
         return torch.cuda.current_stream().cuda_stream
+    return raw(torch._C._cuda_getDevice())
+
+
+def _stream(stream):
+    if stream is None:
+        return _current_raw_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
