@@ -96,6 +96,27 @@ __device__ __forceinline__ uint32_t bins4(const BandDesc &f, const uint8_t *s_lu
   }
 }
 
+// Joint bins of the four pixels of C channels at src, loaded as C words (4 C
+// byte loads, in both roles of the count kernel, cost a 1920x1080 RGB frame 6
+// us: 94.5 -> 88.6).
+template <int C>
+__device__ __forceinline__ uint32_t joint4(const BandDesc &f, const uint8_t *src) {
+  uint32_t v[C], q = 0u;
+#pragma unroll
+  for (int c = 0; c < C; ++c) v[c] = __ldcg(reinterpret_cast<const unsigned int *>(src) + c);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    uint32_t k = 0u;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      const int at = i * C + c;
+      k += ((__byte_perm(v[at >> 2], 0u, 0x4440u + (at & 3)) * (uint32_t)f.jmul[c]) >> 8) * (uint32_t)f.jstride[c];
+    }
+    q |= k << (8 * i);
+  }
+  return q;
+}
+
 // Put the bins of rows r, r + step, .. < nrows (of the rows from y0 on) at
 // columns x .. x+3 into a tile column (and, with to_q, into the plane of
 // bins).  Columns past the frame get bin 0: they lie right of every column
@@ -108,13 +129,25 @@ __device__ __forceinline__ void load_tile(const BandDesc &f, const uint8_t *s_lu
   uint8_t *qp = f.q + (size_t)(y0 + r) * wpad + x;
   const long long sstep = (long long)step * f.pitch;
   const size_t qstep = (size_t)step * wpad;
-  const bool words = MODE != kBinJoint && x + 3 < f.W &&
-                     ((reinterpret_cast<uintptr_t>(f.in) | (uintptr_t)f.pitch) & 3u) == 0;
-  if (words) {
-    src += x;
-#pragma unroll 8
+  if constexpr (MODE == kBinJoint) {
+    const bool words = x + 3 < f.W && ((reinterpret_cast<uintptr_t>(f.in) | (uintptr_t)f.pitch) & 3u) == 0;
+    src += x * f.jc;
+#pragma unroll 2
     for (; r < nrows; r += step) {
-      const uint32_t q = bins4<MODE>(f, s_lut, __ldcg(reinterpret_cast<const unsigned int *>(src)));
+      uint32_t q = 0u;
+      if (words) {
+        q = f.jc == 3 ? joint4<3>(f, src) : f.jc == 4 ? joint4<4>(f, src) : f.jc == 2 ? joint4<2>(f, src) : joint4<1>(f, src);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (x + i < f.W) {
+            uint32_t k = 0u;
+            for (int c = 0; c < f.jc; ++c)
+              k += (((uint32_t)__ldg(src + i * f.jc + c) * (uint32_t)f.jmul[c]) >> 8) * (uint32_t)f.jstride[c];
+            q |= k << (8 * i);
+          }
+        }
+      }
       *tp = q;
       if (to_q) *reinterpret_cast<uint32_t *>(qp) = q;
       src += sstep;
@@ -122,31 +155,32 @@ __device__ __forceinline__ void load_tile(const BandDesc &f, const uint8_t *s_lu
       qp += qstep;
     }
   } else {
+    const bool words = x + 3 < f.W && ((reinterpret_cast<uintptr_t>(f.in) | (uintptr_t)f.pitch) & 3u) == 0;
+    src += x;
+    if (words) {
+#pragma unroll 8
+      for (; r < nrows; r += step) {
+        const uint32_t q = bins4<MODE>(f, s_lut, __ldcg(reinterpret_cast<const unsigned int *>(src)));
+        *tp = q;
+        if (to_q) *reinterpret_cast<uint32_t *>(qp) = q;
+        src += sstep;
+        tp += tstep;
+        qp += qstep;
+      }
+    } else {
 #pragma unroll 2
-    for (; r < nrows; r += step) {
-      uint32_t q = 0u;
-      if constexpr (MODE == kBinJoint) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (x + i < f.W) {
-            uint32_t k = 0u;
-            for (int c = 0; c < f.jc; ++c)
-              k += (((uint32_t)__ldg(src + (x + i) * f.jc + c) * (uint32_t)f.jmul[c]) >> 8) * (uint32_t)f.jstride[c];
-            q |= k << (8 * i);
-          }
-        }
-      } else {
+      for (; r < nrows; r += step) {
         uint32_t v = 0u;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          if (x + i < f.W) v |= (uint32_t)__ldg(src + x + i) << (8 * i);
-        q = bins4<MODE>(f, s_lut, v);
+          if (x + i < f.W) v |= (uint32_t)__ldg(src + i) << (8 * i);
+        const uint32_t q = bins4<MODE>(f, s_lut, v);
+        *tp = q;
+        if (to_q) *reinterpret_cast<uint32_t *>(qp) = q;
+        src += sstep;
+        tp += tstep;
+        qp += qstep;
       }
-      *tp = q;
-      if (to_q) *reinterpret_cast<uint32_t *>(qp) = q;
-      src += sstep;
-      tp += tstep;
-      qp += qstep;
     }
   }
 }

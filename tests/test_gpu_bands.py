@@ -95,6 +95,7 @@ def test_joint_bins(bins):
     for tune in (None, {"overlap": 1}):
         with ihist.Plan(70, 261, bins_per_channel=bins, tune=tune) as plan:
             assert np.array_equal(computed(plan, on_gpu(img, 7, 1)), ref)
+            assert np.array_equal(computed(plan, on_gpu(img, -img[0].size % 4, 4)), ref)  # rows on 4-byte boundaries
 
 
 @pytest.mark.parametrize("layout", [ihist.IHIST_BIN_MAJOR, ihist.IHIST_QUAD_MAJOR, ihist.IHIST_PIXEL_MAJOR])
