@@ -255,7 +255,8 @@ int ihist_query(ihist_plan_t plan, const uint32_t *d_hist, const int32_t *d_rect
  * of bins_per_pass bins reads them bucket by bucket, so the corners of a row
  * share the lines they fall on, and a second pass subtracts each rectangle's
  * upper row from its lower one.
- *   bins_per_pass  bins gathered per pass: 4, 8 or 16 (0 = 8)
+ *   bins_per_pass  bins gathered per pass: 4, 8 or 16 (0 = 16, or 8 for at most
+ *                  8 bins or a d_work that holds no more)
  *   d_work         device scratch of ihist_query_work_bytes(plan, n,
  *                  bins_per_pass) bytes, 256-byte aligned, owned by the
  *                  caller; about 24 + 8 * bins_per_pass bytes per rectangle

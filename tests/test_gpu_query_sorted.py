@@ -107,3 +107,23 @@ def test_sorted_query_row_pairs(nbins, bpp):
         assert plan.status() == ihist.IHIST_OK
     assert np.array_equal(out.cpu().numpy().view(np.uint32), ref)
     assert int(buf[0]) == -3 and bool((buf[1 + len(rects) * nbins:] == -3).all())
+
+
+def test_sorted_query_default_pass_takes_scratch_of_8_bins():
+    h, w, nbins, n = 60, 200, 20, 500
+    img = synth.uniform_frame(29, h, w)
+    rects = synth.rects(31, n, h, w)
+    ref = oracle.query(oracle.integral_histogram(img, nbins), rects)
+    with ihist.Plan(h, w, nbins) as plan:
+        hist = plan.compute(torch.from_numpy(img).cuda())
+        d_rects = torch.from_numpy(rects).cuda()
+        assert plan.query_work_bytes(n) == plan.query_work_bytes(n, 16) > plan.query_work_bytes(n, 8)
+        work = torch.empty((plan.query_work_bytes(n, 8) + 256,), dtype=torch.uint8, device="cuda")
+        out = torch.empty((n, nbins), dtype=torch.int32, device="cuda")
+        need = plan.query_work_bytes(n, 8)
+        work[need:] = 77
+        ihist.ihist_query_sorted(plan.handle, hist.data_ptr(), d_rects.data_ptr(), n, out.data_ptr(), 0,
+                                 work.data_ptr(), need, torch.cuda.current_stream().cuda_stream)
+        assert plan.status() == ihist.IHIST_OK
+    assert np.array_equal(out.cpu().numpy().view(np.uint32), ref)
+    assert bool((work[need:] == 77).all())
