@@ -104,10 +104,12 @@ def time_plan(h, w, nbins, layout, tune, reps=5):
     return statistics.median(ms)
 
 
-def time_batch(shapes, tune, reps=3, tables=False, queries=0):
+def time_batch(shapes, tune, reps=3, tables=False, queries=0, replay=False):
     """Median ms of one batched launch over frames of these (h, w, nbins,
     layout), plus one batched query launch of `queries` rectangles per frame;
-    tables: every frame bins through a value -> bin table."""
+    tables: every frame bins through a value -> bin table.  replay: as a
+    captured graph, which keeps the one-launch form (its work-list is read on
+    the device, so it follows later bindings)."""
     import torch
     frames = [torch.from_numpy(synth.uniform_frame(100 + i, h, w)).cuda() for i, (h, w, b, l) in enumerate(shapes)]
     tb = [[(v * s[2]) >> 8 for v in range(256)] for s in shapes] if tables else None
@@ -127,11 +129,19 @@ def time_batch(shapes, tune, reps=3, tables=False, queries=0):
 
         for _ in range(2):
             step()
+        run = step
+        if replay:
+            graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+            torch.cuda.synchronize()
+            with torch.cuda.graph(graph, stream=side):
+                step()
+            run = graph.replay
+            run()
         ms = []
         for _ in range(reps):
             a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             a.record()
-            step()
+            run()
             b.record()
             torch.cuda.synchronize()
             ms.append(a.elapsed_time(b))
@@ -208,8 +218,9 @@ def tune_batch_layout(shapes, queries_per_frame=0, timer=None, device=None, use_
     """Layout and launch shape of a batch of (h, w, nbins) frames that are
     computed once and then queried `queries_per_frame` times each.  For each
     layout (the same for every frame) the launch shape comes from
-    tune_batch; the layout whose batched launch plus batched queries take
-    less time wins.  timer(shapes, tune, queries) -> ms replaces the
+    tune_batch; the layout whose batched launch plus batched queries,
+    replayed as a graph, take less time wins (live launches of layouts other
+    than bin-major are faster than their replays, not slower).  timer(shapes, tune, queries) -> ms replaces the
     measurement (tests).  Returns (layout, tune, {layout: ms})."""
     device = device or _device_key()
     times, tunes = {}, {}
@@ -221,7 +232,7 @@ def tune_batch_layout(shapes, queries_per_frame=0, timer=None, device=None, use_
         except RuntimeError:
             continue  # no launch shape runs this layout
         times[layout] = (timer(sh, tunes[layout], queries_per_frame) if timer is not None
-                         else time_batch(sh, tunes[layout], queries=queries_per_frame))
+                         else time_batch(sh, tunes[layout], queries=queries_per_frame, replay=True))
     if not times:
         raise RuntimeError("no layout ran")
     layout = min(times, key=times.get)
