@@ -62,7 +62,7 @@ enum {
  * H[b/4][y][x][b%4] at (((b/4)*h + y)*w + x)*4 + b%4 (B a multiple of 4,
  * else IHIST_ERR_INVALID_ARG) -- one 16-byte word per pixel and quad, so a
  * region query reads a quarter of the bin-major layout's DRAM sectors
- * (64 x 1080p x 64: queries 0.25 instead of 0.41 ms, the scan 5.5 instead of
+ * (64 x 1080p x 64: queries 0.25 instead of 0.43 ms, the scan 5.1 against
  * 5.2 ms).  Not a layout of the paper; ihist_window_search does not take
  * it (IHIST_ERR_UNSUPPORTED). */
 enum { IHIST_BIN_MAJOR = 0, IHIST_PIXEL_MAJOR = 1, IHIST_QUAD_MAJOR = 2 };
@@ -122,8 +122,8 @@ typedef struct ihist_plan_s *ihist_plan_t;
  *                   written by the kernel launched just before ihist_compute
  *                   on the same stream (a copy, an event wait or another
  *                   kernel in between makes it safe again).  1080p x 64 per
- *                   frame, back to back: 115 us plain launches, 104 us with
- *                   the default, 99 us with 1.  Joint plans treat 1 as 0
+ *                   frame with 1000 queries: 96 us with the default, 94 with
+ *                   1; 640x480 x 32 the same: 15.7 and 14.4 us.  Joint plans treat 1 as 0
  *                   (their scan reads the joint-bin plane the kernel before
  *                   it writes); ihist_sequence_host always uses 1 (its
  *                   frames arrive by copy).  Batches ignore it.            */
