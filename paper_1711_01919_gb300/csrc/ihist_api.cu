@@ -390,15 +390,8 @@ static int plan_create(int h, int w, int nbins, int layout, const ihist_tune_t *
   if (banded && table && nbins > 252)  // no byte left for "no bin"
     for (int v = 0; v < 256; ++v) banded = banded && bin_map[v] >= 0;
   if (banded) {
-    int optin_b = 0;
-    if (cudaDeviceGetAttribute(&optin_b, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
-      delete p;
-      return IHIST_ERR_CUDA;
-    }
-    const int brc = bands_prepare(band, mode, layout, (size_t)optin_b);
-    if (brc == IHIST_ERR_UNSUPPORTED) {
-      banded = false;
-    } else if (brc != IHIST_OK) {
+    const int brc = bands_prepare(mode, layout);
+    if (brc != IHIST_OK) {
       delete p;
       return brc;
     }

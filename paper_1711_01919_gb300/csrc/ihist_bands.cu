@@ -74,22 +74,21 @@ cudaError_t launch(void (*fn)(const Arg), unsigned int x, unsigned int y, unsign
 }
 
 // Let fn use `smem` bytes of dynamic shared memory.  The attribute belongs to
-// the function, so every plan asks for the same amount: all there is.
+// the function, so every plan asks for the same amount, the most any frame
+// needs.
 template <typename Fn>
-int allow_smem(Fn fn, size_t smem, size_t optin) {
-  cudaFuncAttributes a;
-  if (cudaFuncGetAttributes(&a, fn) != cudaSuccess) {
-    cudaGetLastError();
-    return IHIST_ERR_CUDA;
-  }
-  if (smem + a.sharedSizeBytes > optin) return IHIST_ERR_UNSUPPORTED;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(optin - a.sharedSizeBytes)) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    return IHIST_ERR_CUDA;
-  }
-  return IHIST_OK;
+int allow_smem(Fn fn, size_t smem) {
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) return IHIST_OK;
+  cudaGetLastError();
+  return IHIST_ERR_CUDA;
 }
+
+size_t max_count_smem() {
+  BandDesc f;
+  bands_describe(1, 1, 256, IHIST_BIN_MAJOR, 32, 0, &f);
+  return count_smem_bytes(f);  // 150 KB
+}
+size_t max_emit_smem(int kind) { return kind >= 4 ? pixel_smem_bytes(32) : emit_smem_bytes(kSegWarps, 32); }
 
 }  // namespace
 
@@ -166,10 +165,12 @@ bool bands_shape(int h, int w, int nbins, int layout, int sms, BandDesc *f) {
     R = bands(32) * ctas >= 400 || h > 2048 ? 32 : bands(16) * ctas >= 120 ? 16 : 8;
   }
   bands_describe(h, w, nbins, layout, R, 0, f);
-  // Count threads take R pixels each, or R / 2 where that leaves less than
-  // two CTAs per SM (640x480 x 32: 14.9 -> 14.7 us with its queries; above
-  // it, 1920x1080 x 64, R pixels: 96.4 -> 95.3).
-  if (count_ctas(*f) < 2u * (unsigned)sms) f->split = 1;
+  // Count threads take R pixels each, or R / 2 where that leaves fewer than
+  // 7/4 CTAs per SM, 2 when rows are also counted by strips (1280x720 x 32,
+  // 240 CTAs: 27.3 -> 26.0 us; 1920x1080 with 300 CTAs: x 128 bin-major slower
+  // split, 159.3 -> 162.8, x 64 pixel-major with its queries faster, 108.6 ->
+  // 102).
+  if (4u * count_ctas(*f) < (f->nblk ? 8u : 7u) * (unsigned)sms) f->split = 1;
   return (long long)f->nbands * (f->nblk ? f->nblk : f->nq) * f->nsegs < 0x7fffffffll;
 }
 
@@ -181,19 +182,19 @@ int bands_kind(const BandDesc &f, int layout) {
   return layout == IHIST_QUAD_MAJOR ? (vec ? 2 : 3) : vec && f.W % 4 == 0 ? 0 : 1;
 }
 
-int bands_prepare(const BandDesc &f, int mode, int layout, size_t optin) {
-  int rc = allow_smem(count_fn(mode), count_smem_bytes(f), optin);
+int bands_prepare(int mode, int layout) {
+  int rc = allow_smem(count_fn(mode), max_count_smem());
   for (int kind = 0; kind < kBandKinds && rc == IHIST_OK; ++kind)
-    if (bands_kind_layout(kind) == layout) rc = allow_smem(emit_fn(kind), emit_smem(f, kind), optin);
+    if (bands_kind_layout(kind) == layout) rc = allow_smem(emit_fn(kind), max_emit_smem(kind));
   return rc;
 }
 
-int bands_prepare_batch(size_t optin) {
+int bands_prepare_batch() {
   int rc = IHIST_OK;
   for (int mode = kBinUniform; mode <= kBinJoint && rc == IHIST_OK; ++mode)
-    rc = allow_smem(count_batch_fn(mode), 0, optin);
+    rc = allow_smem(count_batch_fn(mode), max_count_smem());
   for (int kind = 0; kind < kBandKinds && rc == IHIST_OK; ++kind)
-    rc = allow_smem(emit_batch_fn(kind), pixel_smem_bytes(32), optin);
+    rc = allow_smem(emit_batch_fn(kind), max_emit_smem(kind));
   return rc;
 }
 

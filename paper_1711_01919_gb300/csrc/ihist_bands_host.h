@@ -33,9 +33,9 @@ bool bands_shape(int h, int w, int nbins, int layout, int sms, BandDesc *f);
 size_t bands_layout(BandDesc *f, char *base, bool any_layout = false);
 
 // Let the kernels of this binning and layout (or all batch kernels) use the
-// shared memory they need (optin: the largest a CTA may have).
-int bands_prepare(const BandDesc &f, int mode, int layout, size_t optin);
-int bands_prepare_batch(size_t optin);
+// shared memory they need.
+int bands_prepare(int mode, int layout);
+int bands_prepare_batch();
 
 // Both launches of one frame, with programmatic stream serialization.
 int launch_bands(const BandDesc &f, int mode, int layout, void *stream);

@@ -220,7 +220,7 @@ struct ihist_batch_s {
     CUtensorMap *tm;
     unsigned int *end, *bins_end;
     uint32_t *lut;
-    BandDesc *bc, *be;
+    BandDesc *bc, *be;  // behind fd, in its allocation
   } stage_sets[2];
   cudaEvent_t staged[2];
   int stage_cur;
@@ -467,8 +467,6 @@ extern "C" void ihist_batch_destroy(ihist_batch_t b) {
     if (st.end) cudaFreeHost(st.end);
     if (st.bins_end) cudaFreeHost(st.bins_end);
     if (st.lut) cudaFreeHost(st.lut);
-    if (st.bc) cudaFreeHost(st.bc);
-    if (st.be) cudaFreeHost(st.be);
   }
   if (b->ws) cudaFree(b->ws);
   if (prev != b->device && prev >= 0) cudaSetDevice(prev);
@@ -648,7 +646,7 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
 
   // The two-launch path: one band height for all frames, by the rules of
   // single frames on their sum, and room for each frame's counts.
-  b->band_ok = !tiled && bands_prepare_batch((size_t)optin) == IHIST_OK;
+  b->band_ok = !tiled && bands_prepare_batch() == IHIST_OK;
   std::vector<size_t> band_bytes(n, 0);
   if (b->band_ok) {
     auto sum = [&](int R, bool pixel) {
@@ -721,16 +719,17 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
       [&]() {
         for (int i = 0; i < 2; ++i) {
           ihist_batch_s::Staging &st = b->stage_sets[i];
-          if (cudaMallocHost((void **)&st.fd, (size_t)n * sizeof(FrameDesc)) != cudaSuccess ||
+          if (cudaMallocHost((void **)&st.fd, (size_t)n * (sizeof(FrameDesc) + 2 * sizeof(BandDesc))) != cudaSuccess ||
               cudaMallocHost((void **)&st.fdq, (size_t)n * sizeof(FrameDesc)) != cudaSuccess ||
               cudaMallocHost((void **)&st.tm, (size_t)n * sizeof(CUtensorMap)) != cudaSuccess ||
               cudaMallocHost((void **)&st.end, (size_t)n * sizeof(unsigned int)) != cudaSuccess ||
               cudaMallocHost((void **)&st.bins_end, (size_t)n * sizeof(unsigned int)) != cudaSuccess ||
               (lut && cudaMallocHost((void **)&st.lut, (size_t)n * 256 * sizeof(uint32_t)) != cudaSuccess) ||
-              cudaMallocHost((void **)&st.bc, (size_t)n * sizeof(BandDesc)) != cudaSuccess ||
-              cudaMallocHost((void **)&st.be, (size_t)n * sizeof(BandDesc)) != cudaSuccess ||
               cudaEventCreateWithFlags(&b->staged[i], cudaEventDisableTiming) != cudaSuccess)
             return false;
+          static_assert(sizeof(FrameDesc) % alignof(BandDesc) == 0, "bc follows fd");
+          st.bc = reinterpret_cast<BandDesc *>(st.fd + n);
+          st.be = st.bc + n;
         }
         return true;
       }() == false ||
