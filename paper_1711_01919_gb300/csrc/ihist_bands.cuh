@@ -14,8 +14,8 @@
 // 1280x720 x 32 36 -> 26, 1920x1080 x 64 104.9 -> 85.5 (a plain fill of the
 // same bytes takes 78.5), 1921x1081 x 64 160 -> 92, 3840x2160 x 64 355 -> 329;
 // quad-major 1920x1080 x 64 108 -> 90, 1921x1081 x 64 582 -> 116; pixel-major
-// 640x480 x 64 61 -> 24, 1920x1080 x 64 150 -> 95, 1921x1081 x 37 300 -> 77,
-// 3840x2160 x 64 521 -> 350.
+// 640x480 x 64 61 -> 22, 1920x1080 x 64 150 -> 92, 1921x1081 x 37 300 -> 74,
+// 3840x2160 x 64 521 -> 348.
 //
 // Superband: 4 bands of R rows (R = 8, 16 or 32).  A group is 4 bins, packed
 // as the bytes of one word; a chunk is 128 columns.  The count kernel leaves
@@ -713,6 +713,9 @@ __global__ void __launch_bounds__(kSegWarps * 32, LAYOUT == 0 && !VEC ? 3 : 4)
 // lanes at all.  One bin per lane makes twice the warps (1920x1080 x 64: 97
 // us against 104), two keep a record that is no multiple of 32 bytes in one
 // warp's hands, whose stores meet in L2 (1921x1081 x 37: 77 against 111).
+// The loads before the first row are what leaves the stores idle (a chain of
+// several L2 round trips per CTA): two groups' and two rows' loads at a time
+// took 1920x1080 x 64 from 97.8 to 92.1 us, 640x480 x 32 from 16.7 to 14.4.
 constexpr int kPixelBins = 64;                // bins of one CTA at most
 constexpr int kStripCols = 32;
 constexpr size_t kPixelTopBytes = (size_t)kChunk * kPixelBins * 4;
@@ -776,65 +779,110 @@ __device__ __forceinline__ void band_emit_pixel(const BandDesc &f, uint8_t *smem
   uint8_t *tile = smem_raw + kPixelTopBytes + (size_t)4 * f.R * kPixelBins * 2;
   for (int e = threadIdx.x; e < nrows * 8; e += blockDim.x)
     copy_async16(tile + 16 * e, f.q + (size_t)(y0 + (e >> 3)) * wpad + c * kChunk + 16 * (e & 7));
-  // counts left of each strip, per row and bin
-  for (int e = threadIdx.x; e < ng << lr; e += blockDim.x) {
-    const int gi = e >> lr, y = e & (f.R - 1);
-    const uint32_t *p = f.rl + (size_t)(g0 + gi) * hpad + y0 + y;
+  // counts left of each strip, per row and bin: two rows (or groups) per
+  // thread with their loads in flight together
+  const int lefts = ng << lr;
+  for (int e0 = threadIdx.x; e0 < lefts; e0 += 2 * WARPS * 32) {
     const size_t step = (size_t)f.nq * hpad;
-    uint32_t lo = 0u, hi = 0u;
-#pragma unroll 8
-    for (int cl = 0; cl < c; ++cl) add_bytes16(lo, hi, __ldcg(p + cl * step));
-    const uint32_t *ps = f.rls + ((size_t)(3 * c) * f.nq + g0 + gi) * hpad + y0 + y;
+    const bool two = e0 + WARPS * 32 < lefts;
+    const uint32_t *p[2];
+    uint32_t lo[2] = {0u, 0u}, hi[2] = {0u, 0u}, sv[2][3];
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      uint32_t l = lo, h = hi;
-      if (s > 0) add_bytes16(l, h, __ldcg(ps + (s - 1) * step));
-      s_left[(s * f.R + y) * kUnits + (gi ^ (y & 15))] =
-          make_uint2((l & 0xffffu) | h << 16, l >> 16 | (h & 0xffff0000u));
+    for (int u = 0; u < 2; ++u) {
+      const int e = two ? e0 + u * WARPS * 32 : e0;
+      p[u] = f.rl + (size_t)(g0 + (e >> lr)) * hpad + y0 + (e & (f.R - 1));
+      const uint32_t *ps = f.rls + ((size_t)(3 * c) * f.nq + g0 + (e >> lr)) * hpad + y0 + (e & (f.R - 1));
+#pragma unroll
+      for (int i = 0; i < 3; ++i) sv[u][i] = __ldcg(ps + i * step);
     }
-  }
-  // H in the row above the band, four bins of the chunk at a time
-  const int sbk = k / kSuper;
-  for (int gi = w; gi < ng; gi += WARPS) {
-    const int g = g0 + gi;
-    const int x = c * kChunk + 4 * lane;
-    uint32_t lo[4] = {0u, 0u, 0u, 0u}, hi[4] = {0u, 0u, 0u, 0u};
-    auto add = [&](uint4 p) {
-      add_bytes16(lo[0], hi[0], p.x);
-      add_bytes16(lo[1], hi[1], p.y);
-      add_bytes16(lo[2], hi[2], p.z);
-      add_bytes16(lo[3], hi[3], p.w);
-    };
-    const uint32_t *sp = f.sb + (size_t)g * wpad + x;
-    const size_t sstep = (size_t)f.nq * wpad;
 #pragma unroll 4
-    for (int s = 0; s < sbk; ++s) add(__ldcg(reinterpret_cast<const uint4 *>(sp + s * sstep)));
-    if (k % kSuper) add(__ldcg(reinterpret_cast<const uint4 *>(f.pb + ((size_t)k * f.nq + g) * wpad + x)));
-    uint32_t left[4] = {0u, 0u, 0u, 0u};
-    const uint2 *ctp = f.ct + (size_t)g * f.nchunks * f.nbands + lane;
-    for (int j = lane; j < k; j += 32, ctp += 32) {
-#pragma unroll 8
-      for (int cl = 0; cl < c; ++cl) {
-        const uint2 v = __ldcg(ctp + (size_t)cl * f.nbands);
-        left[0] += v.x & 0xffffu;
-        left[2] += v.x >> 16;
-        left[1] += v.y & 0xffffu;
-        left[3] += v.y >> 16;
+    for (int cl = 0; cl < c; ++cl) {
+      const uint32_t v0 = __ldcg(p[0] + cl * step), v1 = __ldcg(p[1] + cl * step);
+      add_bytes16(lo[0], hi[0], v0);
+      add_bytes16(lo[1], hi[1], v1);
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      if (u == 1 && !two) break;
+      const int e = e0 + u * WARPS * 32, gi = e >> lr, y = e & (f.R - 1);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        uint32_t l = lo[u], h = hi[u];
+        if (i > 0) add_bytes16(l, h, sv[u][i - 1]);
+        s_left[(i * f.R + y) * kUnits + (gi ^ (y & 15))] = make_uint2((l & 0xffffu) | h << 16, l >> 16 | (h & 0xffff0000u));
       }
     }
-    uint32_t top[4][4];
+  }
+  // H in the row above the band, four bins of the chunk at a time, two such
+  // groups per warp with their loads in flight together
+  const int sbk = k / kSuper;
+  for (int gi0 = w; gi0 < ng; gi0 += 2 * WARPS) {
+    const bool two = gi0 + WARPS < ng;
+    const int g = g0 + gi0;
+    const int x = c * kChunk + 4 * lane;
+    uint32_t lo[2][4], hi[2][4], left[2][4];
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const uint32_t l = __reduce_add_sync(kFull, left[b]);
+    for (int u = 0; u < 2; ++u)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) top[b][i] = (((b & 1) ? hi[i] : lo[i]) >> (b & 2 ? 16 : 0)) & 0xffffu;
-      chunk_prefix(top[b], lane);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) top[b][i] += l;
+      for (int i = 0; i < 4; ++i) lo[u][i] = hi[u][i] = left[u][i] = 0u;
+    auto add = [&](int u, uint4 p) {
+      add_bytes16(lo[u][0], hi[u][0], p.x);
+      add_bytes16(lo[u][1], hi[u][1], p.y);
+      add_bytes16(lo[u][2], hi[u][2], p.z);
+      add_bytes16(lo[u][3], hi[u][3], p.w);
+    };
+    auto add_left = [&](int u, uint2 v) {
+      left[u][0] += v.x & 0xffffu;
+      left[u][2] += v.x >> 16;
+      left[u][1] += v.y & 0xffffu;
+      left[u][3] += v.y >> 16;
+    };
+    const uint4 none = make_uint4(0u, 0u, 0u, 0u);
+    const size_t sstep = (size_t)f.nq * wpad;
+    const uint32_t *sp = f.sb + (size_t)g * wpad + x, *sp2 = sp + (size_t)WARPS * wpad;
+#pragma unroll 4
+    for (int s = 0; s < sbk; ++s) {
+      const uint4 p0 = __ldcg(reinterpret_cast<const uint4 *>(sp + s * sstep));
+      const uint4 p1 = two ? __ldcg(reinterpret_cast<const uint4 *>(sp2 + s * sstep)) : none;
+      add(0, p0);
+      add(1, p1);
+    }
+    if (k % kSuper) {
+      const uint32_t *pb = f.pb + ((size_t)k * f.nq + g) * wpad + x;
+      const uint4 p0 = __ldcg(reinterpret_cast<const uint4 *>(pb));
+      const uint4 p1 = two ? __ldcg(reinterpret_cast<const uint4 *>(pb + (size_t)WARPS * wpad)) : none;
+      add(0, p0);
+      add(1, p1);
+    }
+    const uint2 *ctp = f.ct + (size_t)g * f.nchunks * f.nbands + lane;
+    const size_t cstep = (size_t)WARPS * f.nchunks * f.nbands;
+    for (int j = lane; j < k; j += 32, ctp += 32) {
+#pragma unroll 4
+      for (int cl = 0; cl < c; ++cl) {
+        const uint2 v0 = __ldcg(ctp + (size_t)cl * f.nbands);
+        const uint2 v1 = two ? __ldcg(ctp + cstep + (size_t)cl * f.nbands) : make_uint2(0u, 0u);
+        add_left(0, v0);
+        add_left(1, v1);
+      }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      s_top[(4 * lane + i) * kUnits + (gi ^ (lane & 7))] = make_uint4(top[0][i], top[1][i], top[2][i], top[3][i]);
+    for (int u = 0; u < 2; ++u) {
+      if (u == 1 && !two) break;
+      const int gi = gi0 + u * WARPS;
+      uint32_t top[4][4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const uint32_t l = __reduce_add_sync(kFull, left[u][b]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) top[b][i] = (((b & 1) ? hi[u][i] : lo[u][i]) >> (b & 2 ? 16 : 0)) & 0xffffu;
+        chunk_prefix(top[b], lane);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) top[b][i] += l;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        s_top[(4 * lane + i) * kUnits + (gi ^ (lane & 7))] = make_uint4(top[0][i], top[1][i], top[2][i], top[3][i]);
+    }
   }
   copy_async_wait();
   __syncthreads();
