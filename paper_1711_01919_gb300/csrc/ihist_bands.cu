@@ -216,11 +216,13 @@ unsigned int bands_threads(const BandDesc &f, int kind) {
 }
 
 // One launch per run of frames of the same kernel, at most kBatchFrames each.
-int launch_bands_batch(const BandRun *runs, int nruns, void *stream) {
+int launch_bands_batch(const BandRun *runs, int nruns, unsigned int stamp, Ctrl *ctrl, void *stream) {
   for (int i = 0; i < nruns; ++i) {
     const BandRun &r = runs[i];
     BandBatch b;
     b.frames = r.d_desc;
+    b.ctrl = ctrl;
+    b.stamp = stamp;
     b.n = r.n;
     unsigned int total = 0;
     size_t smem = 0;

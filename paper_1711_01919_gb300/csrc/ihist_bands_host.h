@@ -42,13 +42,14 @@ int launch_bands(const BandDesc &f, int mode, int layout, void *stream);
 
 // One launch of a batch: n frames (at most kBatchFrames) through the count
 // kernel of a binning or the emit kernel of a kind; their descriptors on the
-// device and on the host.
+// device and on the host.  The descriptors carry the stamp of their binding;
+// CTAs that find another one on the device do nothing but latch the status.
 struct BandRun {
   bool count;
   int kernel, n;
   const BandDesc *d_desc, *h_desc;
 };
-int launch_bands_batch(const BandRun *runs, int nruns, void *stream);
+int launch_bands_batch(const BandRun *runs, int nruns, unsigned int stamp, Ctrl *ctrl, void *stream);
 
 }  // namespace host
 }  // namespace ihist

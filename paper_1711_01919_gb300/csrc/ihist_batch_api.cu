@@ -211,6 +211,7 @@ struct ihist_batch_s {
   BandDesc *d_bc, *d_be;               // descriptors by count kernel and by emit kernel
   std::vector<BandDesc> bc, be;        // the current binding's, in those orders
   std::vector<BandRun> runs;           // its launches; empty: the look-back kernel
+  unsigned int binding;                // bindings so far, the stamp of the current one's descriptors
   // Pinned staging of the descriptors, two sets used by alternate bindings:
   // a binding waits only for the copy made from its set two bindings ago,
   // so a caller can bind and launch ahead of the GPU.  h_* point at the set
@@ -230,6 +231,11 @@ struct ihist_batch_s {
   uint32_t *h_lut;
   cudaEvent_t uploaded, computed;
   bool launched;
+  // The two-launch path's grids come from the binding, so its launches must
+  // find that binding's descriptors: the stream the copies are ordered before
+  // (a launch on another one waits for staged[stage_cur] first, once).
+  void *bound_stream;
+  bool bound_wait;  // false: the copies were made at plan time, or captured into a graph
 };
 
 // TMA descriptor of the plane the scan reads (the frame, or its joint-bin plane).
@@ -276,6 +282,7 @@ static bool bands_bind(ihist_batch_s *b, const ihist_frame_t *frames, const std:
     f.pitch = (long long)fr.in_pitch;
     f.out = fr.d_out;
     f.ctrl = b->ctrl;
+    f.stamp = f.stamp_end = b->binding + 1u;
     mode[i] = kBinUniform;
     if (fr.bin_of_value) {
       mode[i] = kBinTable;
@@ -421,6 +428,7 @@ static int batch_bind(ihist_batch_s *b, const ihist_frame_t *frames, int n) {
   b->fd.assign(fd.begin(), fd.end());
   b->io.assign(frames, frames + n);
   b->n = n;
+  ++b->binding;
   b->tma = tma;
   b->vec = vec;
   b->total = (unsigned int)total;
@@ -811,6 +819,18 @@ extern "C" int ihist_batch_get_tune(ihist_batch_t b, ihist_tune_t *out) {
   return IHIST_OK;
 }
 
+// A captured launch has to follow later bindings when it is replayed.  The
+// look-back launch reads its work-list on the device; the two-launch path's
+// grids are those of the binding at the call, so it is not captured.
+static bool under_capture(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
 extern "C" int ihist_batch_set_io(ihist_batch_t b, const ihist_frame_t *frames, int n, void *stream) {
   if (!b || !frames) return IHIST_ERR_INVALID_ARG;
   int rc = check_batch_device(b);
@@ -826,19 +846,9 @@ extern "C" int ihist_batch_set_io(ihist_batch_t b, const ihist_frame_t *frames, 
     use_staging(b, prev);
     return rc;
   }
+  b->bound_stream = stream;
+  b->bound_wait = !under_capture((cudaStream_t)stream);
   return batch_upload(b, (cudaStream_t)stream);
-}
-
-// A captured launch has to follow later bindings when it is replayed.  The
-// look-back launch reads its work-list on the device; the two-launch path's
-// grids are those of the binding at the call, so it is not captured.
-static bool under_capture(cudaStream_t s) {
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
-    cudaGetLastError();
-    return true;
-  }
-  return st != cudaStreamCaptureStatusNone;
 }
 
 extern "C" int ihist_batch_compute(ihist_batch_t b, void *stream) {
@@ -846,7 +856,11 @@ extern "C" int ihist_batch_compute(ihist_batch_t b, void *stream) {
   int rc = check_batch_device(b);
   if (rc != IHIST_OK) return rc;
   if (!b->runs.empty() && !under_capture((cudaStream_t)stream)) {
-    rc = launch_bands_batch(b->runs.data(), (int)b->runs.size(), stream);
+    if (b->bound_wait && stream != b->bound_stream) {
+      if (cudaStreamWaitEvent((cudaStream_t)stream, b->staged[b->stage_cur], 0) != cudaSuccess) return IHIST_ERR_CUDA;
+      b->bound_stream = stream;
+    }
+    rc = launch_bands_batch(b->runs.data(), (int)b->runs.size(), b->binding, b->ctrl, stream);
     if (rc != IHIST_OK) return rc;
     if (cudaEventRecord(b->computed, (cudaStream_t)stream) != cudaSuccess) return IHIST_ERR_CUDA;
     b->launched = true;
