@@ -93,8 +93,6 @@ size_t max_emit_smem(int kind) { return kind >= 4 ? pixel_smem_bytes(32) : emit_
 }  // namespace
 
 size_t bands_layout(BandDesc *f, char *base, bool any_layout) {
-  const size_t wpad = (size_t)f->nchunks * kChunk;
-  const size_t hpad = (size_t)f->nsb * kSuper * f->R;
   const bool pixel = f->nblk > 0;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -102,13 +100,12 @@ size_t bands_layout(BandDesc *f, char *base, bool any_layout) {
     off = align_up(off + bytes, 256);
     return p;
   };
-  f->q = reinterpret_cast<uint8_t *>(take((size_t)f->H * wpad));
-  f->pb = reinterpret_cast<uint32_t *>(take((size_t)f->nbands * f->nq * wpad * 4));
-  f->sb = reinterpret_cast<uint32_t *>(take((size_t)f->nsb * f->nq * wpad * 4));
-  f->rl = reinterpret_cast<uint32_t *>(take((size_t)f->nchunks * f->nq * hpad * 4));
-  f->ct = reinterpret_cast<uint2 *>(
-      take(f->nsegs > 1 || any_layout ? (size_t)f->nbands * f->nq * f->nchunks * 8 : 0));
-  f->rls = reinterpret_cast<uint32_t *>(take(pixel || any_layout ? (size_t)f->nchunks * 3 * f->nq * hpad * 4 : 0));
+  f->q = reinterpret_cast<uint8_t *>(take(q_size(*f)));
+  f->pb = reinterpret_cast<uint32_t *>(take(pb_size(*f) * 4));
+  f->sb = reinterpret_cast<uint32_t *>(take(sb_size(*f) * 4));
+  f->rl = reinterpret_cast<uint32_t *>(take(rl_size(*f) * 4));
+  f->ct = reinterpret_cast<uint2 *>(take(f->nsegs > 1 || any_layout ? ct_size(*f) * 8 : 0));
+  f->rls = reinterpret_cast<uint32_t *>(take(pixel || any_layout ? rls_size(*f) * 4 : 0));
   if (!pixel) f->rls = nullptr;
   return off;
 }

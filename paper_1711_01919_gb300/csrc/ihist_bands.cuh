@@ -64,6 +64,17 @@ struct BandDesc {
   unsigned int stamp_end;
 };
 
+// Elements of the workspace's arrays.
+__host__ __device__ inline size_t q_size(const BandDesc &f) { return (size_t)f.H * f.nchunks * kChunk; }
+__host__ __device__ inline size_t pb_size(const BandDesc &f) { return (size_t)f.nbands * f.nq * f.nchunks * kChunk; }
+__host__ __device__ inline size_t sb_size(const BandDesc &f) { return (size_t)f.nsb * f.nq * f.nchunks * kChunk; }
+__host__ __device__ inline size_t rl_size(const BandDesc &f) { return (size_t)f.nchunks * f.nq * f.nsb * kSuper * f.R; }
+__host__ __device__ inline size_t rls_size(const BandDesc &f) { return 3 * rl_size(f); }
+__host__ __device__ inline size_t ct_size(const BandDesc &f) { return (size_t)f.nbands * f.nq * f.nchunks; }
+
+// Checked builds: whether the n elements at p lie in array a of the workspace.
+#define IHIST_IN(f, a, p, n) IHIST_GUARD((f).ctrl, (p) >= (f).a && (p) + (n) <= (f).a + a##_size(f))
+
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -151,7 +162,7 @@ __device__ __forceinline__ void load_tile(const BandDesc &f, const uint8_t *s_lu
         }
       }
       *tp = q;
-      if (to_q) *reinterpret_cast<uint32_t *>(qp) = q;
+      if (to_q && IHIST_IN(f, q, qp, 4)) *reinterpret_cast<uint32_t *>(qp) = q;
       src += sstep;
       tp += tstep;
       qp += qstep;
@@ -164,7 +175,7 @@ __device__ __forceinline__ void load_tile(const BandDesc &f, const uint8_t *s_lu
       for (; r < nrows; r += step) {
         const uint32_t q = bins4<MODE>(f, s_lut, __ldcg(reinterpret_cast<const unsigned int *>(src)));
         *tp = q;
-        if (to_q) *reinterpret_cast<uint32_t *>(qp) = q;
+        if (to_q && IHIST_IN(f, q, qp, 4)) *reinterpret_cast<uint32_t *>(qp) = q;
         src += sstep;
         tp += tstep;
         qp += qstep;
@@ -178,7 +189,7 @@ __device__ __forceinline__ void load_tile(const BandDesc &f, const uint8_t *s_lu
           if (x + i < f.W) v |= (uint32_t)__ldg(src + i) << (8 * i);
         const uint32_t q = bins4<MODE>(f, s_lut, v);
         *tp = q;
-        if (to_q) *reinterpret_cast<uint32_t *>(qp) = q;
+        if (to_q && IHIST_IN(f, q, qp, 4)) *reinterpret_cast<uint32_t *>(qp) = q;
         src += sstep;
         tp += tstep;
         qp += qstep;
@@ -211,6 +222,10 @@ __host__ __device__ inline size_t count_smem_bytes(const BandDesc &f) {
 template <int MODE>
 __device__ __forceinline__ void band_count(const BandDesc &f, uint8_t *smem_raw, const uint3 block) {
   __shared__ uint8_t s_lut[MODE == kBinTable ? 256 : 1];
+  if (!IHIST_GUARD(f.ctrl, block.x < 2u * f.nchunks && (int)block.y * col_tile_rows(f) < f.H && block.z < 2u)) {
+    griddep_wait();
+    return;
+  }
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   uint32_t *tile32 = reinterpret_cast<uint32_t *>(smem_raw);
   uint32_t *hist = reinterpret_cast<uint32_t *>(smem_raw + count_tile_bytes(f));
@@ -243,7 +258,7 @@ __device__ __forceinline__ void band_count(const BandDesc &f, uint8_t *smem_raw,
       const uint32_t *rp = tile32 + tcol;
       uint8_t *qp = f.q + (size_t)(y0 + (t >> 4)) * wpad + x4;
       for (int r = t >> 4; r < nrows; r += kRowStep, rp += kTileStep, qp += kRowStep * wpad)
-        *reinterpret_cast<uint32_t *>(qp) = *rp;
+        if (IHIST_IN(f, q, qp, 4)) *reinterpret_cast<uint32_t *>(qp) = *rp;
     }
     __syncthreads();
     const int x = t & (kHalf - 1), piece = t / kHalf;
@@ -281,9 +296,10 @@ __device__ __forceinline__ void band_count(const BandDesc &f, uint8_t *smem_raw,
 #pragma unroll
         for (int j = 1; j < kSuper; ++j) {
           pb += band_step;
-          if (j < nbk) *pb = above[j];
+          if (j < nbk && IHIST_IN(f, pb, pb, 1)) *pb = above[j];
         }
-        f.sb[(size_t)sb * band_step + at] = above[kSuper];
+        uint32_t *sbp = f.sb + (size_t)sb * band_step + at;
+        if (IHIST_IN(f, sb, sbp, 1)) *sbp = above[kSuper];
       }
     }
   } else {
@@ -328,12 +344,12 @@ __device__ __forceinline__ void band_count(const BandDesc &f, uint8_t *smem_raw,
             for (int p = 0; p < kCountThreads; p += trows) {
               n += hg[p];
               if (((p + trows) & strip) == 0 && p + trows < kCountThreads) {
-                *rls = n;
+                if (IHIST_IN(f, rls, rls, 1)) *rls = n;
                 rls += (size_t)f.nq * hpad;
               }
             }
           }
-          *rl = n;
+          if (IHIST_IN(f, rl, rl, 1)) *rl = n;
         }
         if (f.nsegs > 1) {
           // a band's R rows lie in neighbouring lanes
@@ -347,7 +363,7 @@ __device__ __forceinline__ void band_count(const BandDesc &f, uint8_t *smem_raw,
               hi += __shfl_xor_sync(kFull, hi, d);
             }
           }
-          if (in && first) *ct = make_uint2(lo, hi);
+          if (in && first && IHIST_IN(f, ct, ct, 1)) *ct = make_uint2(lo, hi);
           ct += (size_t)pieces * f.nchunks * f.nbands;
         }
         hg += pieces * kCountThreads;
@@ -483,6 +499,7 @@ __device__ __forceinline__ void band_emit(const BandDesc &f, uint8_t *smem_raw, 
   const int k = (int)(planes ? it % (unsigned)f.nbands : it / ngs);
   const int c0 = seg * f.cps;
   const int c = c0 + w - w0;
+  if (!IHIST_GUARD(f.ctrl, k < f.nbands && gs < f.nq && c0 < f.nchunks)) return;
   const bool live = lg < f.gpc && g < f.nq && c < f.nchunks;
   const int y0 = k * f.R;
   const int nrows = min(f.R, f.H - y0);
@@ -494,14 +511,18 @@ __device__ __forceinline__ void band_emit(const BandDesc &f, uint8_t *smem_raw, 
   uint32_t acc[4][4];  // running H of this lane's 4 columns, per bin
   if (live) {
     const uint8_t *qp = f.q + (size_t)y0 * wpad + c * kChunk;
-    for (int r = lane >> 3; r < nrows; r += 4)
-      copy_async16(tile + r * kChunk + 16 * (lane & 7), qp + (size_t)r * wpad + 16 * (lane & 7));
-    const uint32_t own = lane < f.R ? __ldcg(f.rl + ((size_t)c * f.nq + g) * hpad + y0 + lane) : 0u;
+    for (int r = lane >> 3; r < nrows; r += 4) {
+      const uint8_t *src = qp + (size_t)r * wpad + 16 * (lane & 7);
+      if (IHIST_IN(f, q, src, 16)) copy_async16(tile + r * kChunk + 16 * (lane & 7), src);
+    }
+    const uint32_t *rp = f.rl + ((size_t)c * f.nq + g) * hpad + y0 + lane;
+    const uint32_t own = lane < f.R && IHIST_IN(f, rl, rp, 1) ? __ldcg(rp) : 0u;
     // counts above the band in this lane's columns, two bins per word
     uint32_t lo[4], hi[4];
     {
-      const uint4 p = k % kSuper ? __ldcg(reinterpret_cast<const uint4 *>(f.pb + ((size_t)k * f.nq + g) * wpad + x))
-                                 : make_uint4(0u, 0u, 0u, 0u);  // a superband's first band
+      const uint32_t *pp = f.pb + ((size_t)k * f.nq + g) * wpad + x;
+      const uint4 p = k % kSuper && IHIST_IN(f, pb, pp, 4) ? __ldcg(reinterpret_cast<const uint4 *>(pp))
+                                                           : make_uint4(0u, 0u, 0u, 0u);  // a superband's first band
       const uint32_t pv[4] = {p.x, p.y, p.z, p.w};
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -513,6 +534,7 @@ __device__ __forceinline__ void band_emit(const BandDesc &f, uint8_t *smem_raw, 
     const size_t sstep = (size_t)f.nq * wpad;
 #pragma unroll 4
     for (int s = 0; s < sbk; ++s) {
+      if (!IHIST_IN(f, sb, sp + s * sstep, 4)) break;
       const uint4 p = __ldcg(reinterpret_cast<const uint4 *>(sp + s * sstep));
       add_bytes16(lo[0], hi[0], p.x);
       add_bytes16(lo[1], hi[1], p.y);
@@ -534,8 +556,10 @@ __device__ __forceinline__ void band_emit(const BandDesc &f, uint8_t *smem_raw, 
     // the chunks left of the segment, shared out over the CTA's warps (which
     // hold one group then)
     uint2 l = make_uint2(0u, 0u);
-    for (int cl = w; cl < c0; cl += nw)
-      if (lane < f.R) add_bytes16(l.x, l.y, __ldcg(f.rl + ((size_t)cl * f.nq + gs) * hpad + y0 + lane));
+    for (int cl = w; cl < c0; cl += nw) {
+      const uint32_t *rp = f.rl + ((size_t)cl * f.nq + gs) * hpad + y0 + lane;
+      if (lane < f.R && IHIST_IN(f, rl, rp, 1)) add_bytes16(l.x, l.y, __ldcg(rp));
+    }
     s_left[w][lane] = l;
     uint4 tot = make_uint4(0u, 0u, 0u, 0u);
     auto add = [&](uint2 v) {
@@ -546,7 +570,10 @@ __device__ __forceinline__ void band_emit(const BandDesc &f, uint8_t *smem_raw, 
     };
 #pragma unroll 4
     for (int cl = w; cl < c0; cl += nw)
-      for (int j = lane; j < k; j += 32) add(__ldcg(f.ct + ((size_t)gs * f.nchunks + cl) * f.nbands + j));
+      for (int j = lane; j < k; j += 32) {
+        const uint2 *cp = f.ct + ((size_t)gs * f.nchunks + cl) * f.nbands + j;
+        if (IHIST_IN(f, ct, cp, 1)) add(__ldcg(cp));
+      }
     tot.x = __reduce_add_sync(kFull, tot.x);
     tot.y = __reduce_add_sync(kFull, tot.y);
     tot.z = __reduce_add_sync(kFull, tot.z);
@@ -794,8 +821,11 @@ __device__ __forceinline__ void band_emit_pixel(const BandDesc &f, uint8_t *smem
   const size_t hpad = (size_t)f.nsb * kSuper * f.R;
   const int lr = __ffs(f.R) - 1;
   uint8_t *tile = smem_raw + kPixelTopBytes + (size_t)4 * f.R * kPixelBins * 2;
-  for (int e = threadIdx.x; e < nrows * 8; e += blockDim.x)
-    copy_async16(tile + 16 * e, f.q + (size_t)(y0 + (e >> 3)) * wpad + c * kChunk + 16 * (e & 7));
+  if (!IHIST_GUARD(f.ctrl, k < f.nbands)) return;
+  for (int e = threadIdx.x; e < nrows * 8; e += blockDim.x) {
+    const uint8_t *src = f.q + (size_t)(y0 + (e >> 3)) * wpad + c * kChunk + 16 * (e & 7);
+    if (IHIST_IN(f, q, src, 16)) copy_async16(tile + 16 * e, src);
+  }
   // counts left of each strip, per row and bin: two rows (or groups) per
   // thread with their loads in flight together
   const int lefts = ng << lr;
@@ -810,10 +840,11 @@ __device__ __forceinline__ void band_emit_pixel(const BandDesc &f, uint8_t *smem
       p[u] = f.rl + (size_t)(g0 + (e >> lr)) * hpad + y0 + (e & (f.R - 1));
       const uint32_t *ps = f.rls + ((size_t)(3 * c) * f.nq + g0 + (e >> lr)) * hpad + y0 + (e & (f.R - 1));
 #pragma unroll
-      for (int i = 0; i < 3; ++i) sv[u][i] = __ldcg(ps + i * step);
+      for (int i = 0; i < 3; ++i) sv[u][i] = IHIST_IN(f, rls, ps + i * step, 1) ? __ldcg(ps + i * step) : 0u;
     }
 #pragma unroll 4
     for (int cl = 0; cl < c; ++cl) {
+      if (!IHIST_IN(f, rl, p[0] + cl * step, 1) || !IHIST_IN(f, rl, p[1] + cl * step, 1)) break;
       const uint32_t v0 = __ldcg(p[0] + cl * step), v1 = __ldcg(p[1] + cl * step);
       add_bytes16(lo[0], hi[0], v0);
       add_bytes16(lo[1], hi[1], v1);
@@ -859,13 +890,14 @@ __device__ __forceinline__ void band_emit_pixel(const BandDesc &f, uint8_t *smem
     const uint32_t *sp = f.sb + (size_t)g * wpad + x, *sp2 = sp + (size_t)WARPS * wpad;
 #pragma unroll 4
     for (int s = 0; s < sbk; ++s) {
+      if (!IHIST_IN(f, sb, sp + s * sstep, 4) || (two && !IHIST_IN(f, sb, sp2 + s * sstep, 4))) break;
       const uint4 p0 = __ldcg(reinterpret_cast<const uint4 *>(sp + s * sstep));
       const uint4 p1 = two ? __ldcg(reinterpret_cast<const uint4 *>(sp2 + s * sstep)) : none;
       add(0, p0);
       add(1, p1);
     }
-    if (k % kSuper) {
-      const uint32_t *pb = f.pb + ((size_t)k * f.nq + g) * wpad + x;
+    const uint32_t *pb = f.pb + ((size_t)k * f.nq + g) * wpad + x;
+    if (k % kSuper && IHIST_IN(f, pb, pb, 4) && (!two || IHIST_IN(f, pb, pb + (size_t)WARPS * wpad, 4))) {
       const uint4 p0 = __ldcg(reinterpret_cast<const uint4 *>(pb));
       const uint4 p1 = two ? __ldcg(reinterpret_cast<const uint4 *>(pb + (size_t)WARPS * wpad)) : none;
       add(0, p0);
@@ -876,6 +908,9 @@ __device__ __forceinline__ void band_emit_pixel(const BandDesc &f, uint8_t *smem
     for (int j = lane; j < k; j += 32, ctp += 32) {
 #pragma unroll 4
       for (int cl = 0; cl < c; ++cl) {
+        if (!IHIST_IN(f, ct, ctp + (size_t)cl * f.nbands, 1) ||
+            (two && !IHIST_IN(f, ct, ctp + cstep + (size_t)cl * f.nbands, 1)))
+          break;
         const uint2 v0 = __ldcg(ctp + (size_t)cl * f.nbands);
         const uint2 v1 = two ? __ldcg(ctp + cstep + (size_t)cl * f.nbands) : make_uint2(0u, 0u);
         add_left(0, v0);
