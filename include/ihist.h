@@ -127,7 +127,11 @@ typedef struct ihist_plan_s *ihist_plan_t;
  *                   1; 640x480 x 32 the same: 15.7 and 14.4 us.  Joint plans treat 1 as 0
  *                   (their scan reads the joint-bin plane the kernel before
  *                   it writes); ihist_sequence_host always uses 1 (its
- *                   frames arrive by copy).  Batches ignore it.            */
+ *                   frames arrive by copy).  Batches ignore it.
+ *   reserved        0; ihist_plan_get_tune and ihist_batch_get_tune report 1
+ *                   there if the plan, or the batch with its current binding,
+ *                   takes the two-launch path (captured batch launches never
+ *                   do).  Ignored when passed in.                          */
 typedef struct {
   int rows_per_band;
   int bins_per_cta;

@@ -600,6 +600,7 @@ extern "C" int ihist_plan_get_tune(ihist_plan_t p, ihist_tune_t *out) {
   out->groups_per_cta = p->gpc;
   out->warps_per_cta = p->NW;
   out->overlap = p->overlap;
+  out->reserved = p->banded ? 1 : 0;
   return IHIST_OK;
 }
 

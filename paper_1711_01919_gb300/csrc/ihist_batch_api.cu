@@ -816,6 +816,7 @@ extern "C" int ihist_batch_get_tune(ihist_batch_t b, ihist_tune_t *out) {
   out->fault_skip_band = b->fault_skip_band + 1;  // 0 = off
   out->groups_per_cta = 0;  // chosen per frame
   out->warps_per_cta = b->warps;
+  out->reserved = b->runs.empty() ? 0 : 1;
   return IHIST_OK;
 }
 

@@ -257,6 +257,13 @@ def ihist_plan_get_tune(plan: int) -> dict:
     return {k: getattr(t, k) for k in TUNE_FIELDS}
 
 
+def two_launch_plan(plan: int) -> bool:
+    """Whether the plan's frames take the two-launch path."""
+    t = ihist_tune_t()
+    _check(load().ihist_plan_get_tune(plan, ctypes.byref(t)), "ihist_plan_get_tune")
+    return t.reserved == 1
+
+
 def ihist_workspace_bytes(plan: int) -> int:
     return int(load().ihist_workspace_bytes(plan))
 
@@ -387,6 +394,13 @@ def ihist_batch_get_tune(batch: int) -> dict:
     t = ihist_tune_t()
     _check(load().ihist_batch_get_tune(batch, ctypes.byref(t)), "ihist_batch_get_tune")
     return {k: getattr(t, k) for k in TUNE_FIELDS}
+
+
+def two_launch_batch(batch: int) -> bool:
+    """Whether launches of the batch's binding (not captured) take the two-launch path."""
+    t = ihist_tune_t()
+    _check(load().ihist_batch_get_tune(batch, ctypes.byref(t)), "ihist_batch_get_tune")
+    return t.reserved == 1
 
 
 def ihist_batch_set_io(batch: int, frames, stream: int = 0) -> None:
