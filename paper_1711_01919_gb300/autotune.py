@@ -13,7 +13,8 @@ are multiples of 4) quad-major output and keep the fastest, for callers
 that accept any.
 
 Results are cached in a JSON file (``IHIST_TUNE_CACHE`` or
-``~/.cache/ihist_tune.json``) keyed by device name and shape.  The timing
+``~/.cache/ihist_tune.json``) keyed by device name, shape and (batches) launch
+form, with the set of kernels they were measured against.  The timing
 function is injectable, so the search and cache logic run on the CPU in the
 tests.
 """
@@ -28,6 +29,12 @@ from . import ihist, synth
 
 _lock = threading.Lock()
 
+# The kernels that an untuned call may take.  A cached tiling is used only if
+# it was measured against the same set (a tiling keeps plans and batches on the
+# look-back kernel, so one found before the two-launch path existed would pin
+# calls to the slower of the two).
+KERNELS = "look-back, two-launch"
+
 
 def cache_path() -> str:
     return os.environ.get("IHIST_TUNE_CACHE") or os.path.join(os.path.expanduser("~"), ".cache", "ihist_tune.json")
@@ -39,6 +46,20 @@ def _load_cache(path):
             return json.load(f)
     except (OSError, ValueError):
         return {}
+
+
+def _cached_tune(path, key):
+    """The cached tiling of a key, or None."""
+    with _lock:
+        entry = _load_cache(path).get(key)
+    return entry["tune"] if isinstance(entry, dict) and entry.get("kernels") == KERNELS else None
+
+
+def _remember(path, key, tune, ms):
+    with _lock:
+        cache = _load_cache(path)
+        cache[key] = {"tune": tune, "ms": ms, "kernels": KERNELS}
+        _store_cache(path, cache)
 
 
 def _store_cache(path, cache):
@@ -108,7 +129,7 @@ def time_batch(shapes, tune, reps=3, tables=False, queries=0, replay=False):
     """Median ms of one batched launch over frames of these (h, w, nbins,
     layout), plus one batched query launch of `queries` rectangles per frame;
     tables: every frame bins through a value -> bin table.  replay: as a
-    captured graph, which keeps the one-launch form (its work-list is read on
+    captured graph, which keeps the look-back kernel (its work-list is read on
     the device, so it follows later bindings)."""
     import torch
     frames = [torch.from_numpy(synth.uniform_frame(100 + i, h, w)).cuda() for i, (h, w, b, l) in enumerate(shapes)]
@@ -170,38 +191,33 @@ def tune_plan(h, w, nbins, layout=ihist.IHIST_BIN_MAJOR, timer=None, device=None
     device = device or _device_key()
     key = "plan|%s|%dx%dx%d|%d" % (device, h, w, nbins, layout)
     path = cache_path()
-    with _lock:
-        cache = _load_cache(path) if use_cache else {}
-        if key in cache:
-            return cache[key]["tune"]
+    cached = _cached_tune(path, key) if use_cache else None
+    if cached is not None:
+        return cached
     timer = timer or (lambda t: time_plan(h, w, nbins, layout, t))
     best, ms, _ = _search(plan_candidates(h, w, nbins), timer)
     if use_cache:
-        with _lock:
-            cache = _load_cache(path)
-            cache[key] = {"tune": best, "ms": ms}
-            _store_cache(path, cache)
+        _remember(path, key, best, ms)
     return best
 
 
-def tune_batch(shapes, timer=None, device=None, use_cache=True, tables=False):
+def tune_batch(shapes, timer=None, device=None, use_cache=True, tables=False, replay=False):
     """Best (warps_per_cta, bins_per_cta, rows_per_band) for a batch of (h, w,
-    nbins, layout) frames; tables: a table batch (other bin structures)."""
+    nbins, layout) frames; tables: a table batch (other bin structures).
+    replay: for launches replayed from a captured graph, which never take the
+    two-launch path that an untuned live launch may take."""
     device = device or _device_key()
     sig = ",".join("%dx%dx%dx%d" % tuple(s) for s in sorted(set(tuple(s) for s in shapes)))
     key = "batch|%s|%d|%s%s" % (device, len(shapes), sig, "|tables" if tables else "")
+    key += "|replay" if replay else ""
     path = cache_path()
-    with _lock:
-        cache = _load_cache(path) if use_cache else {}
-        if key in cache:
-            return cache[key]["tune"]
-    timer = timer or (lambda t: time_batch(shapes, t, tables=tables))
+    cached = _cached_tune(path, key) if use_cache else None
+    if cached is not None:
+        return cached
+    timer = timer or (lambda t: time_batch(shapes, t, tables=tables, replay=replay))
     best, ms, _ = _search(batch_candidates(shapes, tables), timer)
     if use_cache:
-        with _lock:
-            cache = _load_cache(path)
-            cache[key] = {"tune": best, "ms": ms}
-            _store_cache(path, cache)
+        _remember(path, key, best, ms)
     return best
 
 
@@ -214,25 +230,27 @@ def layouts_for(nbins_list):
     return out
 
 
-def tune_batch_layout(shapes, queries_per_frame=0, timer=None, device=None, use_cache=True):
+def tune_batch_layout(shapes, queries_per_frame=0, timer=None, device=None, use_cache=True, replay=False):
     """Layout and launch shape of a batch of (h, w, nbins) frames that are
     computed once and then queried `queries_per_frame` times each.  For each
     layout (the same for every frame) the launch shape comes from
-    tune_batch; the layout whose batched launch plus batched queries,
-    replayed as a graph, take less time wins (live launches of layouts other
-    than bin-major are faster than their replays, not slower).  timer(shapes, tune, queries) -> ms replaces the
-    measurement (tests).  Returns (layout, tune, {layout: ms})."""
+    tune_batch; the layout whose batched launch plus batched queries take less
+    time wins.  Launch shapes and layouts are compared in the form the caller
+    will use: live launches, or (replay) graph replays.  timer(shapes, tune,
+    queries) -> ms replaces the measurement (tests).  Returns (layout, tune,
+    {layout: ms})."""
     device = device or _device_key()
     times, tunes = {}, {}
     for layout in layouts_for([b for (h, w, b) in shapes]):
         sh = [(h, w, b, layout) for (h, w, b) in shapes]
         shape_timer = None if timer is None else (lambda t, sh=sh: timer(sh, t, 0))
         try:
-            tunes[layout] = tune_batch(sh, timer=shape_timer, device=device, use_cache=use_cache)
+            tunes[layout] = tune_batch(sh, timer=shape_timer, device=device, use_cache=use_cache,
+                                      replay=replay)
         except RuntimeError:
             continue  # no launch shape runs this layout
         times[layout] = (timer(sh, tunes[layout], queries_per_frame) if timer is not None
-                         else time_batch(sh, tunes[layout], queries=queries_per_frame, replay=True))
+                         else time_batch(sh, tunes[layout], queries=queries_per_frame, replay=replay))
     if not times:
         raise RuntimeError("no layout ran")
     layout = min(times, key=times.get)
