@@ -212,6 +212,18 @@ unsigned int bands_threads(const BandDesc &f, int kind) {
   return kind == 5 ? 256u : kind >= 4 ? 128u : 32u * (unsigned)(f.wpg * f.gpc);
 }
 
+// A count launch gives every CTA the shared memory of its largest frame, and
+// shared memory is what limits its CTAs per SM (up to 72 bins four, 108 three,
+// 180 two, above that one, at 32 rows per band), so frames share a launch only
+// with frames that allow as many (where they are more than a few waves): 255
+// frames of 320x240 x 8 and one of x 256, with their emit launch, took 268 us
+// in one launch and take 182 in two, 31 of 1280x720 x 32 and one of x 256 810
+// and 740.
+int bands_count_class(const BandDesc &f) {
+  constexpr size_t kSm = 228u << 10, kOther = 2048;  // an SM's shared memory; static and reserved bytes of a CTA
+  return (int)std::min<size_t>(4, kSm / (count_smem_bytes(f) + kOther));
+}
+
 // One launch per run of frames of the same kernel, at most kBatchFrames each.
 int launch_bands_batch(const BandRun *runs, int nruns, unsigned int stamp, Ctrl *ctrl, void *stream) {
   for (int i = 0; i < nruns; ++i) {

@@ -40,6 +40,9 @@ int bands_prepare_batch();
 // Both launches of one frame, with programmatic stream serialization.
 int launch_bands(const BandDesc &f, int mode, int layout, void *stream);
 
+// Count CTAs per SM that a frame's shared memory allows (1..4).
+int bands_count_class(const BandDesc &f);
+
 // One launch of a batch: n frames (at most kBatchFrames) through the count
 // kernel of a binning or the emit kernel of a kind; their descriptors on the
 // device and on the host.  The descriptors carry the stamp of their binding;

@@ -270,7 +270,9 @@ static bool bands_bind(ihist_batch_s *b, const ihist_frame_t *frames, const std:
   }
   if (!other && plain > (16ull << 30)) return false;
   std::vector<BandDesc> desc(n);
-  std::vector<int> mode(n), kind(n), order(n);
+  std::vector<int> count(n), kind(n), order(n);  // kernels of each frame: binning and CTAs per SM, emit kind
+  int least = 4;                // CTAs per SM of one launch for all
+  unsigned long long ctas = 0;  // and its CTAs
   for (int i = 0; i < n; ++i) {
     const ihist_frame_t &fr = frames[i];
     if (!bands_fit(fr.h, fr.w, fr.layout)) return false;
@@ -283,15 +285,15 @@ static bool bands_bind(ihist_batch_s *b, const ihist_frame_t *frames, const std:
     f.out = fr.d_out;
     f.ctrl = b->ctrl;
     f.stamp = f.stamp_end = b->binding + 1u;
-    mode[i] = kBinUniform;
+    int mode = kBinUniform;
     if (fr.bin_of_value) {
-      mode[i] = kBinTable;
+      mode = kBinTable;
       f.lut = fd[i].lut;
       if (fr.nbins > 252)  // no byte left for "no bin"
         for (int v = 0; v < 256; ++v)
           if (fr.bin_of_value[v] < 0) return false;
     } else if (frame_joint(fr)) {
-      mode[i] = kBinJoint;
+      mode = kBinJoint;
       f.jc = fr.channels;
       int stride = 1;
       for (int c = fr.channels - 1; c >= 0; --c) {
@@ -300,14 +302,21 @@ static bool bands_bind(ihist_batch_s *b, const ihist_frame_t *frames, const std:
         stride *= f.jmul[c];
       }
     }
+    count[i] = 4 * mode + bands_count_class(f) - 1;
+    least = std::min(least, count[i] % 4 + 1);
+    ctas += count_ctas(f);
     kind[i] = bands_kind(f, fr.layout);
     order[i] = i;
   }
+  // One launch where it is a few waves at most (7 frames of 640x480 x 16 and
+  // one of x 128: 56 us in one, 64 in two).
+  if (ctas <= 4ull * least * b->sms)
+    for (int &c : count) c -= c % 4;
   bc->clear();
   be->clear();
   runs->clear();
   for (int pass = 0; pass < 2; ++pass) {
-    const std::vector<int> &key = pass ? kind : mode;
+    const std::vector<int> &key = pass ? kind : count;
     std::vector<BandDesc> *to = pass ? be : bc;
     // by kernel, then largest first, so that a launch ends on small frames
     std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
@@ -317,10 +326,9 @@ static bool bands_bind(ihist_batch_s *b, const ihist_frame_t *frames, const std:
     });
     for (int i = 0; i < n; ++i) {
       to->push_back(desc[order[i]]);
-      const int kernel = key[order[i]];
-      if (i == 0 || runs->back().count != (pass == 0) || runs->back().kernel != kernel ||
-          runs->back().n == kBatchFrames)
-        runs->push_back(BandRun{pass == 0, kernel, 0, (pass ? b->d_be : b->d_bc) + i, nullptr});
+      const int k = key[order[i]];
+      if (i == 0 || k != key[order[i - 1]] || runs->back().n == kBatchFrames)
+        runs->push_back(BandRun{pass == 0, pass ? k : k / 4, 0, (pass ? b->d_be : b->d_bc) + i, nullptr});
       ++runs->back().n;
     }
   }
