@@ -144,16 +144,27 @@ bool bands_fit(int h, int w, int layout) {
   return h <= 8192 && (long long)h * w <= (layout == IHIST_BIN_MAJOR ? 12000000ll : 40000000ll);
 }
 
+// Rows per band: long bands write fewer counts, short ones make more warps
+// (each emits one chunk of one band).  640x480 x 32 at R = 8, 16, 32: 11.6,
+// 11.3, 11.4 us; 320x240 x 16: 5.7, 6.9, 9.2; 1920x1080 x 64 with 1000
+// queries behind it: 106, 95, 103; 3840x2160 x 64: 488, 343, 329.  Where pixels
+// are many and bins few, there are not that many warps, but the count kernel is
+// what takes the time, and it is the faster the more pixels share a thread's
+// counters: at R = 16 and 32 12000x1000 x 4 takes 62 and 57 us, 65532x183 x 8
+// 121 and 98, 24 frames of 1920x1080 x 1 188 and 137, 64 of 640x480 x 4 98 and
+// 85 (below that, the order changes with the last wave: 2400x2000 x 8 44 and 47,
+// 16 frames of 640x480 x 12 51 and 59, x 4 28 and 26).
+int bands_rows(long long warps32, long long warps16, long long pixels, int h_max) {
+  if (warps32 >= 16000 || h_max > 2048 || pixels >= 11000000) return 32;
+  return warps16 >= 600 ? 16 : 8;
+}
+
 bool bands_shape(int h, int w, int nbins, int layout, int sms, BandDesc *f) {
   if (!bands_fit(h, w, layout)) return false;
   bands_describe(h, w, nbins, layout, 32, 0, f);
-  // Rows per band: long bands write fewer counts, short ones make more warps
-  // (each emits one chunk of one band).  640x480 x 32 at R = 8, 16, 32: 11.6,
-  // 11.3, 11.4 us; 320x240 x 16: 5.7, 6.9, 9.2; 1920x1080 x 64 with 1000
-  // queries behind it: 106, 95, 103; 3840x2160 x 64: 488, 343, 329.
   const long long per_band = (long long)f->nq * f->nchunks;
   auto bands = [&](int R) { return (long long)((h + R - 1) / R); };
-  int R = bands(32) * per_band >= 16000 || h > 2048 ? 32 : bands(16) * per_band >= 600 ? 16 : 8;
+  int R = bands_rows(bands(32) * per_band, bands(16) * per_band, (long long)h * w, h);
   if (layout == IHIST_PIXEL_MAJOR) {
     // by CTAs: 1920x1080 x 64 at R = 32 (510 CTAs) and 16: 97, 100 us; 640x480
     // x 64 at 32, 16 (150 CTAs) and 8: 27.8, 23.9, 25.8; 320x240 x 16 at 16

@@ -22,6 +22,10 @@ unsigned int bands_threads(const BandDesc &f, int kind);
 // Whether the two-launch path is the faster one for a frame of this size.
 bool bands_fit(int h, int w, int layout);
 
+// Rows per band of bin- or quad-major frames: emit warps at 32 and 16 rows per
+// band, pixels, and the tallest frame.
+int bands_rows(long long warps32, long long warps16, long long pixels, int h_max);
+
 // The shape fields of a frame with R rows per band.
 void bands_describe(int h, int w, int nbins, int layout, int R, int split, BandDesc *f);
 

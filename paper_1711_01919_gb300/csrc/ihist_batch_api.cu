@@ -677,9 +677,12 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
     };
     int h_max = 0;
     for (int i = 0; i < n; ++i) h_max = std::max(h_max, frames[i].h);
-    b->band_R = sum(32, false) >= 16000 || sum(32, true) >= 400 || h_max > 2048 ? 32
-                : sum(16, false) >= 600 || sum(16, true) >= 120                 ? 16
-                                                                                : 8;
+    long long px = 0;
+    for (int i = 0; i < n; ++i)
+      if (frames[i].layout != IHIST_PIXEL_MAJOR) px += (long long)frames[i].h * frames[i].w;
+    b->band_R = bands_rows(sum(32, false), sum(16, false), px, h_max);
+    if (sum(32, true) >= 400) b->band_R = 32;
+    else if (sum(16, true) >= 120) b->band_R = std::max(b->band_R, 16);
     unsigned long long ctas = 0;
     for (int i = 0; i < n; ++i) {
       BandDesc f;
