@@ -250,7 +250,7 @@ static int plan_create(int h, int w, int nbins, int layout, const ihist_tune_t *
   const bool tiled = t.rows_per_band || t.bins_per_cta || t.chunks_per_warp || t.ctas_per_sm || t.groups_per_cta ||
                      t.warps_per_cta || t.fault_skip_band >= 1;
   BandDesc band;
-  bool banded = !tiled && bands_shape(h, w, nbins, layout, sms, &band);
+  bool banded = !tiled && bands_shape(h, w, nbins, layout, table, sms, &band);
   // Pixel-major output: a pixel's counts of one bin group are G contiguous
   // words and the groups of a pixel belong to different CTAs, so larger
   // groups give longer contiguous pieces per pixel record; rows are staged

@@ -159,7 +159,32 @@ int bands_rows(long long warps32, long long warps16, long long pixels, int h_max
   return warps16 >= 600 ? 16 : 8;
 }
 
-bool bands_shape(int h, int w, int nbins, int layout, int sms, BandDesc *f) {
+// Frames within those sizes that the look-back kernel still does faster.
+static bool look_back_faster(const BandDesc &f, int layout, bool table) {
+  const long long px = (long long)f.H * f.W;
+  if (layout == IHIST_PIXEL_MAJOR)
+    // records of one or two whole sectors, which that kernel stores complete:
+    // 4320x7680 x 8 440 us against 460 here, 400x65532 x 8 and x 16 1.16x and
+    // 1.07x faster (x 12 0.8x; here a CTA also adds up the counts of all chunks
+    // to its left), 4320x5800 x 8 0.94x
+    return (f.B == 8 && px > (f.W > 48000 ? 16000000 : 30000000)) ||
+           (f.B == 16 && f.W > 62000 && px > 24000000);
+  // Bins and counts that L2 does not hold, where its own loads are whole (rows
+  // of 16-byte multiples): bin-major 3840x2160 x 128 (58 MB) 660 us here, 663
+  // there, x 192 (83 MB) 998 / 967, 3200x2500 x 160 (68 MB) 788 / 808, 4000x3000
+  // x 64 (48 MB) 483 / 487, x 256 (156 MB) 1960 / 1820; in one CTA a band (up to 16 chunks) 1456x8192 x 160 (101
+  // MB) the same, x 192 1.03x; quad-major 7680x4320 x 96 (182 MB) 0.99x, x 128
+  // (232 MB) 1.02x, 4800x8192 x 192 5743 / 4986.  Rows of other widths are
+  // faster here at any size (1464x8192 x 256 0.79x).  With tables, which cost
+  // that kernel more, the lines lie higher (bin-major 4000x3000 x 128 the same,
+  // x 192 1.03x, quad-major 4800x8192 x 128 0.97x, x 192 1.06x).
+  const long long mb = layout == IHIST_QUAD_MAJOR ? (table ? 335 : 190)
+                       : f.nchunks > 16           ? (table ? 110 : 72)
+                                                  : (table ? 160 : 105);
+  return f.W % 16 == 0 && (long long)(q_size(f) + 4 * (pb_size(f) + sb_size(f) + rl_size(f))) > mb * 1000000;
+}
+
+bool bands_shape(int h, int w, int nbins, int layout, bool table, int sms, BandDesc *f) {
   if (!bands_fit(h, w, layout)) return false;
   bands_describe(h, w, nbins, layout, 32, 0, f);
   const long long per_band = (long long)f->nq * f->nchunks;
@@ -173,6 +198,7 @@ bool bands_shape(int h, int w, int nbins, int layout, int sms, BandDesc *f) {
     R = bands(32) * ctas >= 400 || h > 2048 ? 32 : bands(16) * ctas >= 120 ? 16 : 8;
   }
   bands_describe(h, w, nbins, layout, R, 0, f);
+  if (look_back_faster(*f, layout, table)) return false;
   // Count threads take R pixels each, or R / 2 where that leaves fewer than
   // 7/4 CTAs per SM, 2 when rows are also counted by strips (1280x720 x 32,
   // 240 CTAs: 27.3 -> 26.0 us; 1920x1080 with 300 CTAs: x 128 bin-major slower

@@ -29,8 +29,9 @@ int bands_rows(long long warps32, long long warps16, long long pixels, int h_max
 // The shape fields of a frame with R rows per band.
 void bands_describe(int h, int w, int nbins, int layout, int R, int split, BandDesc *f);
 
-// Whether a plan's frames take the two-launch path, and their shape in *f.
-bool bands_shape(int h, int w, int nbins, int layout, int sms, BandDesc *f);
+// Whether a plan's frames take the two-launch path, and their shape in *f
+// (table: they bin through a value -> bin table).
+bool bands_shape(int h, int w, int nbins, int layout, bool table, int sms, BandDesc *f);
 
 // Workspace bytes of the shape; with a base (256-byte aligned), also the
 // pointers into it.  any_layout: enough for the same shape in every layout.
