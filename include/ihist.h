@@ -50,9 +50,8 @@ enum {
   IHIST_ERR_CUDA = 4,             /* a CUDA runtime call failed */
   IHIST_ERR_LOOKBACK_TIMEOUT = 5, /* device: a carry wait ran out of time (result invalid) */
   IHIST_ERR_BAD_RECT = 6,         /* device: a query rectangle was out of range (its row is zero) */
-  IHIST_ERR_CHECK_FAILED = 7      /* device: an access that could not be right was skipped (result invalid): a
-                                     batch's descriptors on the device were not those of the launched binding,
-                                     or, in checked builds, an index was out of range (a library bug) */
+  IHIST_ERR_CHECK_FAILED = 7      /* device, checked builds only: an out-of-range access was caught and
+                                     skipped (result invalid; a library bug) */
 };
 
 /* Output layouts of H.  Bin-major is the paper's b x h x w tensor mapped
@@ -421,11 +420,9 @@ int ihist_batch_get_tune(ihist_batch_t batch, ihist_tune_t *out);
  * Nothing is allocated. */
 int ihist_batch_set_io(ihist_batch_t batch, const ihist_frame_t *frames, int n, void *stream);
 
-/* Compute every bound frame of the batch in one launch on `stream`.  A launch
- * on another stream than the binding's waits for the binding's copies.  Where
- * a later binding's copies, on yet another stream, overtake a launch that has
- * not run, that launch may write nothing and latch IHIST_ERR_CHECK_FAILED: the
- * caller orders ihist_batch_set_io after the launches it must not disturb. */
+/* Compute every bound frame of the batch in one launch on `stream`.  Bindings
+ * and launches may be on different streams: a live launch of the two-launch
+ * path runs after its binding's copies, and a later binding's copies after it. */
 int ihist_batch_compute(ihist_batch_t batch, void *stream);
 
 /* Region histograms (Eq. 2) on frame `frame` of the batch; arguments as for

@@ -262,13 +262,11 @@ int bands_count_class(const BandDesc &f) {
 }
 
 // One launch per run of frames of the same kernel, at most kBatchFrames each.
-int launch_bands_batch(const BandRun *runs, int nruns, unsigned int stamp, Ctrl *ctrl, void *stream) {
+int launch_bands_batch(const BandRun *runs, int nruns, void *stream) {
   for (int i = 0; i < nruns; ++i) {
     const BandRun &r = runs[i];
     BandBatch b;
     b.frames = r.d_desc;
-    b.ctrl = ctrl;
-    b.stamp = stamp;
     b.n = r.n;
     unsigned int total = 0;
     size_t smem = 0;

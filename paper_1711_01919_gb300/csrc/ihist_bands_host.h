@@ -50,14 +50,13 @@ int bands_count_class(const BandDesc &f);
 
 // One launch of a batch: n frames (at most kBatchFrames) through the count
 // kernel of a binning or the emit kernel of a kind; their descriptors on the
-// device and on the host.  The descriptors carry the stamp of their binding;
-// CTAs that find another one on the device do nothing but latch the status.
+// device and on the host.  The launch must find these descriptors on the device.
 struct BandRun {
   bool count;
   int kernel, n;
   const BandDesc *d_desc, *h_desc;
 };
-int launch_bands_batch(const BandRun *runs, int nruns, unsigned int stamp, Ctrl *ctrl, void *stream);
+int launch_bands_batch(const BandRun *runs, int nruns, void *stream);
 
 }  // namespace host
 }  // namespace ihist

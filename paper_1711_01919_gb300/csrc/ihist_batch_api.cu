@@ -211,7 +211,6 @@ struct ihist_batch_s {
   BandDesc *d_bc, *d_be;               // descriptors by count kernel and by emit kernel
   std::vector<BandDesc> bc, be;        // the current binding's, in those orders
   std::vector<BandRun> runs;           // its launches; empty: the look-back kernel
-  unsigned int binding;                // bindings so far, the stamp of the current one's descriptors
   // Pinned staging of the descriptors, two sets used by alternate bindings:
   // a binding waits only for the copy made from its set two bindings ago,
   // so a caller can bind and launch ahead of the GPU.  h_* point at the set
@@ -229,13 +228,19 @@ struct ihist_batch_s {
   CUtensorMap *h_tm;
   unsigned int *h_end, *h_bins_end;
   uint32_t *h_lut;
-  cudaEvent_t uploaded, computed;
+  cudaEvent_t uploaded;
+  // The last launch's completion: `banded` after a launch of the two-launch path
+  // (never captured), `computed` after one of the look-back kernel.
+  cudaEvent_t computed, banded, last;
   bool launched;
-  // The two-launch path's grids come from the binding, so its launches must
-  // find that binding's descriptors: the stream the copies are ordered before
-  // (a launch on another one waits for staged[stage_cur] first, once).
-  void *bound_stream;
-  bool bound_wait;  // false: the copies were made at plan time, or captured into a graph
+  // A two-launch launch has its binding's CTA counts and reads its descriptors
+  // on the device, so it must run between that binding's copies and the next
+  // one's.  bound_stream: the stream the copies are on (a launch on another one
+  // waits for staged[stage_cur] first, once; bound_wait false: they were made at
+  // plan time).  banded_stream: the stream of the last such launch (copies and
+  // launches on another one wait for it).
+  void *bound_stream, *banded_stream;
+  bool bound_wait, banded_wait;
 };
 
 // TMA descriptor of the plane the scan reads (the frame, or its joint-bin plane).
@@ -284,7 +289,6 @@ static bool bands_bind(ihist_batch_s *b, const ihist_frame_t *frames, const std:
     f.pitch = (long long)fr.in_pitch;
     f.out = fr.d_out;
     f.ctrl = b->ctrl;
-    f.stamp = f.stamp_end = b->binding + 1u;
     int mode = kBinUniform;
     if (fr.bin_of_value) {
       mode = kBinTable;
@@ -436,7 +440,6 @@ static int batch_bind(ihist_batch_s *b, const ihist_frame_t *frames, int n) {
   b->fd.assign(fd.begin(), fd.end());
   b->io.assign(frames, frames + n);
   b->n = n;
-  ++b->binding;
   b->tma = tma;
   b->vec = vec;
   b->total = (unsigned int)total;
@@ -475,6 +478,7 @@ extern "C" void ihist_batch_destroy(ihist_batch_t b) {
   }
   if (b->uploaded) cudaEventDestroy(b->uploaded);
   if (b->computed) cudaEventDestroy(b->computed);
+  if (b->banded) cudaEventDestroy(b->banded);
   for (int i = 0; i < 2; ++i) {
     ihist_batch_s::Staging &st = b->stage_sets[i];
     if (st.fd) cudaFreeHost(st.fd);
@@ -753,7 +757,8 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
         return true;
       }() == false ||
       cudaEventCreateWithFlags(&b->uploaded, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&b->computed, cudaEventDisableTiming) != cudaSuccess) {
+      cudaEventCreateWithFlags(&b->computed, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&b->banded, cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
     ihist_batch_destroy(b);
     return IHIST_ERR_OOM;
@@ -858,9 +863,25 @@ extern "C" int ihist_batch_set_io(ihist_batch_t b, const ihist_frame_t *frames, 
     use_staging(b, prev);
     return rc;
   }
+  // The copies follow the launches that read the descriptors they replace.
+  // Captured copies are made when the graph is replayed: until the next binding
+  // launches go through the look-back kernel, which takes what it finds.  So
+  // they do after copies that failed.
+  if (under_capture((cudaStream_t)stream)) {
+    b->runs.clear();
+    return batch_upload(b, (cudaStream_t)stream);
+  }
+  if (b->banded_wait && stream != b->banded_stream &&
+      cudaStreamWaitEvent((cudaStream_t)stream, b->banded, 0) != cudaSuccess) {
+    b->runs.clear();
+    return IHIST_ERR_CUDA;
+  }
+  b->banded_wait = false;
   b->bound_stream = stream;
-  b->bound_wait = !under_capture((cudaStream_t)stream);
-  return batch_upload(b, (cudaStream_t)stream);
+  b->bound_wait = true;
+  rc = batch_upload(b, (cudaStream_t)stream);
+  if (rc != IHIST_OK) b->runs.clear();
+  return rc;
 }
 
 extern "C" int ihist_batch_compute(ihist_batch_t b, void *stream) {
@@ -872,10 +893,15 @@ extern "C" int ihist_batch_compute(ihist_batch_t b, void *stream) {
       if (cudaStreamWaitEvent((cudaStream_t)stream, b->staged[b->stage_cur], 0) != cudaSuccess) return IHIST_ERR_CUDA;
       b->bound_stream = stream;
     }
-    rc = launch_bands_batch(b->runs.data(), (int)b->runs.size(), b->binding, b->ctrl, stream);
+    if (b->banded_wait && stream != b->banded_stream &&
+        cudaStreamWaitEvent((cudaStream_t)stream, b->banded, 0) != cudaSuccess)
+      return IHIST_ERR_CUDA;
+    rc = launch_bands_batch(b->runs.data(), (int)b->runs.size(), stream);
     if (rc != IHIST_OK) return rc;
-    if (cudaEventRecord(b->computed, (cudaStream_t)stream) != cudaSuccess) return IHIST_ERR_CUDA;
-    b->launched = true;
+    if (cudaEventRecord(b->banded, (cudaStream_t)stream) != cudaSuccess) return IHIST_ERR_CUDA;
+    b->banded_stream = stream;
+    b->banded_wait = b->launched = true;
+    b->last = b->banded;
     return IHIST_OK;
   }
   // joint frames: their joint-bin planes first (the scan waits for them)
@@ -895,6 +921,7 @@ extern "C" int ihist_batch_compute(ihist_batch_t b, void *stream) {
   if (cudaGetLastError() != cudaSuccess) return IHIST_ERR_CUDA;
   if (cudaEventRecord(b->computed, (cudaStream_t)stream) != cudaSuccess) return IHIST_ERR_CUDA;
   b->launched = true;
+  b->last = b->computed;
   return IHIST_OK;
 }
 
@@ -907,7 +934,7 @@ extern "C" int ihist_batch_upload_compute(ihist_batch_t b, const uint8_t *const 
   if (rc != IHIST_OK) return rc;
   cudaStream_t s = (cudaStream_t)stream, cs = (cudaStream_t)copy_stream;
   // inputs are overwritten only after the previous compute of this batch read them
-  if (b->launched && cudaStreamWaitEvent(cs, b->computed, 0) != cudaSuccess) return IHIST_ERR_CUDA;
+  if (b->launched && cudaStreamWaitEvent(cs, b->last, 0) != cudaSuccess) return IHIST_ERR_CUDA;
   for (int i = 0; i < b->n; ++i) {
     const ihist_frame_t &fr = b->io[i];
     const size_t row = (size_t)fr.w * frame_channels(fr);

@@ -1,7 +1,7 @@
 """Batches whose bindings and launches are on different streams.  A launch's
 grid comes from the binding it was made for, its descriptors from device
-memory: a launch waits for its binding's copies wherever they were queued, and
-one that a later binding's copies overtake does nothing but latch the status."""
+memory, so it runs after its binding's copies and before the next binding's,
+wherever these were queued."""
 import numpy as np
 import pytest
 
@@ -66,21 +66,54 @@ def test_a_launch_waits_for_its_bindings_copies(first, second):
 
 
 @pytest.mark.parametrize("first,second", [(SMALL, LARGE), (LARGE, SMALL)])
-def test_a_launch_that_the_next_bindings_copies_overtake_is_refused(first, second):
+def test_the_next_bindings_copies_wait_for_a_launch(first, second):
     imgs, dev, outs = bound(second, 40)
-    _, old_dev, old_outs = bound(first, 50)
+    old_imgs, old_dev, old_outs = bound(first, 50)
     _, slots, slot_outs = bound(LARGE, 60)
-    side = torch.cuda.Stream()
+    side, third = torch.cuda.Stream(), torch.cuda.Stream()
     with ihist.Batch(slots, [s[2] for s in LARGE], [s[3] for s in LARGE], outs=slot_outs) as batch:
         batch.set_io(old_dev, old_outs, [s[2] for s in first], [s[3] for s in first])
         torch.cuda.synchronize()
         torch.cuda._sleep(HOLD)
-        batch.compute()  # has not run when the next binding's copies are made
+        batch.compute()  # has not run when the next binding is made
         batch.set_io(dev, outs, [s[2] for s in second], [s[3] for s in second], stream=side)
-        side.synchronize()
         assert not torch.cuda.current_stream().query()
-        assert batch.status() == ihist.IHIST_ERR_CHECK_FAILED
-        assert all(int((o != -1).sum()) == 0 for o in outs)  # that binding has not been launched
+        batch.compute(stream=third)
+        batch.compute(stream=side)
+        torch.cuda.synchronize()
+        assert batch.status() == ihist.IHIST_OK
+        assert exact(old_imgs, old_outs, first) and exact(imgs, outs, second)
+
+
+def test_upload_compute_on_other_streams_follows_the_last_launch():
+    specs = LARGE
+    imgs, dev, outs = bound(specs, 70)
+    new = [torch.from_numpy(synth.gradient_frame(80 + i, h, w)).pin_memory() for i, (h, w, b, l) in enumerate(specs)]
+    side, copy = torch.cuda.Stream(), torch.cuda.Stream()
+    with ihist.Batch(dev, [s[2] for s in specs], [s[3] for s in specs], outs=outs) as batch:
+        torch.cuda._sleep(HOLD)
+        batch.compute()  # reads the frames that the upload below replaces
+        batch.set_io(dev, [torch.empty_like(o) for o in outs], [s[2] for s in specs], [s[3] for s in specs])
+        batch.upload_compute(new, stream=side, copy_stream=copy)
+        torch.cuda.synchronize()
+        assert batch.status() == ihist.IHIST_OK
+        assert exact(imgs, outs, specs)
+        assert exact([x.numpy() for x in new], batch.outs, specs)
+
+
+def test_a_captured_binding_leaves_live_launches_to_the_look_back_kernel():
+    imgs, dev, outs = bound(LARGE, 90)
+    s_imgs, s_dev, s_outs = bound(SMALL, 95)
+    side = torch.cuda.Stream()
+    with ihist.Batch(dev, [s[2] for s in LARGE], [s[3] for s in LARGE], outs=outs) as batch:
+        batch.compute()
+        torch.cuda.synchronize()
+        assert ihist.two_launch_batch(batch.handle)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side, capture_error_mode="relaxed"):  # it waits for an event on the host
+            batch.set_io(s_dev, s_outs, [s[2] for s in SMALL], [s[3] for s in SMALL])
+        assert not ihist.two_launch_batch(batch.handle)
+        graph.replay()
         batch.compute()
         assert batch.status() == ihist.IHIST_OK
-        assert exact(imgs, outs, second)
+        assert exact(imgs, outs, LARGE) and exact(s_imgs, s_outs, SMALL)
