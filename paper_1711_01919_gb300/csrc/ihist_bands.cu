@@ -172,12 +172,13 @@ static bool look_back_faster(const BandDesc &f, int layout, bool table) {
   // Bins and counts that L2 does not hold, where its own loads are whole (rows
   // of 16-byte multiples): bin-major 3840x2160 x 128 (58 MB) 660 us here, 663
   // there, x 192 (83 MB) 998 / 967, 3200x2500 x 160 (68 MB) 788 / 808, 4000x3000
-  // x 64 (48 MB) 483 / 487, x 256 (156 MB) 1960 / 1820; in one CTA a band (up to 16 chunks) 1456x8192 x 160 (101
-  // MB) the same, x 192 1.03x; quad-major 7680x4320 x 96 (182 MB) 0.99x, x 128
-  // (232 MB) 1.02x, 4800x8192 x 192 5743 / 4986.  Rows of other widths are
-  // faster here at any size (1464x8192 x 256 0.79x).  With tables, which cost
-  // that kernel more, the lines lie higher (bin-major 4000x3000 x 128 the same,
-  // x 192 1.03x, quad-major 4800x8192 x 128 0.97x, x 192 1.06x).
+  // x 64 (48 MB) 483 / 487, x 256 (156 MB) 1960 / 1820; up to 16 chunks wide
+  // 1456x8192 x 160 (101 MB) the same, x 192 1.03x; quad-major 7680x4320 x 96
+  // (182 MB) 0.99x, x 128 (232 MB) 1.02x, 4800x8192 x 192 5743 / 4986.  Rows of
+  // other widths are faster here at any size (1464x8192 x 256 0.79x).  With
+  // tables, which cost that kernel more, the lines lie higher (bin-major
+  // 4000x3000 x 128 the same, x 192 1.03x, quad-major 4800x8192 x 128 0.97x, x
+  // 192 1.06x).
   const long long mb = layout == IHIST_QUAD_MAJOR ? (table ? 335 : 190)
                        : f.nchunks > 16           ? (table ? 110 : 72)
                                                   : (table ? 160 : 105);

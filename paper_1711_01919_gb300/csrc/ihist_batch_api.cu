@@ -256,24 +256,65 @@ static bool encode_frame_map(const uint8_t *in, size_t pitch, int h, int w, int 
              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Whether the look-back kernel is the faster one for a whole batch.  Frames of
+// odd widths or unaligned buffers store better in two launches at any size (8
+// frames of 1921x1080 735 us against 1680); for the others:
+//  - Large bin-major batches hide that kernel's chain behind their stores: 8, 16
+//    and 64 frames of 1920x1080 x 64 take 666, 1316 and 5227 us in two launches
+//    against 722, 1365 and 5210 (32 quad-major ones 2549 against 2791, 8
+//    pixel-major 708 / 1051).
+//  - With few bins, counting takes as long as storing, and it is a pass of its
+//    own here, so from some number of pixels on that kernel is faster (two
+//    launches against one, us): 24 frames of 1920x1080 x 4 214 / 205, 128 of
+//    640x480 x 4 171 / 157, 64 of 1920x1080 x 2 1.11x, x 4 565 / 457, x 8 885 /
+//    800, x 6 (two bins of the second group to write) 1.04x, x 12 1.06x, x 16 1.03x, x 24 1.01x, but 16 of them x 4 0.93x, 24 x 8
+//    0.99x.  It takes about twice as many where frames are wider than 16 chunks,
+//    which fill that kernel's CTAs less evenly (3840x2160 x 4: 6, 12 and 32
+//    frames 0.98x, 1.05x, 1.24x, x 8: 12 and 32 0.98x, 1.09x).  Quad-major:
+//    1920x1080 x 4 24 frames 1.04x, 64 1.20x, x 8 32 0.99x, 64 1.05x, x 12 1.01x.
+//    Pixel-major rows of at most 8 bins leave lanes idle here: 1920x1080 x 4 16
+//    and 24 frames 0.97x and 1.08x, x 8 8 and 24 0.95x and 1.18x, 1921x1081 (rows
+//    that kernel does not load by TMA) x 4 8 and 32 1.04x and 1.09x, x 8 32 and 64
+//    1.01x and 1.05x; up to 1280 columns, where that kernel is at its worst, two
+//    launches stay faster (128 of 1280x720 x 8 0.99x, of 640x480 0.6x).  With
+//    tables the same (24 of 1920x1080 x 4 1.10x, 64 x 8 bin-major 1.12x,
+//    pixel-major 1.20x).
+static bool look_back_faster(const ihist_frame_t *frames, int n) {
+  long long bytes = 0, px = 0, px_bins = 0, wide = 0;
+  int pixel = 0, quad = 0, most = 0, narrow = INT_MAX;
+  bool joint = false, tma = true;
+  for (int i = 0; i < n; ++i) {
+    const ihist_frame_t &fr = frames[i];
+    const long long p = (long long)fr.h * fr.w;
+    if (fr.layout != IHIST_PIXEL_MAJOR && !frame_vec_ok(fr)) return false;
+    joint = joint || frame_joint(fr);
+    tma = tma && frame_tma_ok(fr);
+    pixel += fr.layout == IHIST_PIXEL_MAJOR;
+    quad += fr.layout == IHIST_QUAD_MAJOR;
+    bytes += 4 * p * fr.nbins;
+    px += p;
+    px_bins += p * fr.nbins;
+    if (fr.w > 16 * kChunk) wide += p;
+    most = std::max(most, fr.nbins);
+    narrow = std::min(narrow, fr.w);
+  }
+  if (!pixel && !quad && bytes > (16ll << 30)) return true;
+  if (joint) return false;  // two passes there too
+  const double mean = (double)px_bins / px, mp = px / 1e6;
+  if (pixel)
+    return pixel == n && most <= 8 && narrow > 1280 && mp > (most > 6 ? (tma ? 20 : 60) : (tma ? 36 : 14));
+  if (!tma) return false;
+  const double limit = mean <= 1 ? 180 : mean <= 2 ? 90 : mean <= 4 ? 36 : quad == n ? (mean <= 8 ? 120 : 1e9)
+                       : mean <= 6.5 ? 120 : mean <= 8 ? 64 : mean <= 12 ? 100 : mean <= 16 ? 128 : 1e9;
+  return mp > (2 * wide > px ? 2 * limit : limit);
+}
+
 // Describe the frames for the two-launch path, in launch order; false if one
 // of them does not take it or does not fit its slot.
 static bool bands_bind(ihist_batch_s *b, const ihist_frame_t *frames, const std::vector<FrameDesc> &fd, int n,
                        std::vector<BandDesc> *bc, std::vector<BandDesc> *be, std::vector<BandRun> *runs) {
   if (!b->band_ok) return false;
-  // Large bin-major batches with aligned rows hide the look-back kernel's
-  // chain behind their stores: 8, 16 and 64 frames of 1920x1080 x 64 take
-  // 666, 1316 and 5227 us here against 722, 1365 and 5210 there.  Other
-  // layouts and odd widths store better here at any size (32 quad-major
-  // frames 2549 against 2791 us, 8 pixel-major 708 / 1051, 8 of 1921x1080
-  // 735 / 1680).
-  size_t plain = 0;
-  bool other = false;
-  for (int i = 0; i < n; ++i) {
-    plain += ihist_output_bytes(frames[i].h, frames[i].w, frames[i].nbins);
-    other = other || frames[i].layout != IHIST_BIN_MAJOR || !frame_vec_ok(frames[i]);
-  }
-  if (!other && plain > (16ull << 30)) return false;
+  if (look_back_faster(frames, n)) return false;
   std::vector<BandDesc> desc(n);
   std::vector<int> count(n), kind(n), order(n);  // kernels of each frame: binning and CTAs per SM, emit kind
   int least = 4;                // CTAs per SM of one launch for all

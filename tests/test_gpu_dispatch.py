@@ -44,3 +44,34 @@ def test_plans(h, w, nbins, layout, two):
 def test_table_plans(h, w, nbins, two):
     with ihist.Plan(h, w, nbins, bin_of_value=[v * nbins // 256 for v in range(256)]) as plan:
         assert ihist.two_launch_plan(plan.handle) == two
+
+
+@pytest.mark.parametrize("n,h,w,nbins,layout,two", [
+    # output bytes of aligned bin-major frames
+    (32, 1080, 1920, 64, BIN, True), (33, 1080, 1920, 64, BIN, False), (33, 1080, 1920, 64, QUAD, True),
+    # pixels of frames with few bins, by layout and width
+    (16, 1080, 1920, 4, BIN, True), (24, 1080, 1920, 4, BIN, False), (24, 1080, 1921, 4, BIN, True),
+    (24, 1080, 1928, 4, BIN, True), (24, 1080, 1920, 8, BIN, True), (40, 1080, 1920, 8, BIN, False),
+    (64, 1080, 1920, 16, BIN, False), (64, 1080, 1920, 20, BIN, True), (8, 2160, 3840, 4, BIN, True),
+    (12, 2160, 3840, 4, BIN, False), (40, 1080, 1920, 8, QUAD, True), (64, 1080, 1920, 8, QUAD, False),
+    (9, 1080, 1920, 8, PIXEL, True), (12, 1080, 1920, 8, PIXEL, False), (16, 1080, 1920, 4, PIXEL, True),
+    (24, 1080, 1920, 4, PIXEL, False), (64, 1080, 1920, 9, PIXEL, True), (128, 720, 1280, 8, PIXEL, True),
+    (6, 1081, 1921, 4, PIXEL, True), (8, 1081, 1921, 4, PIXEL, False), (24, 1081, 1921, 8, PIXEL, True),
+])
+def test_batches(n, h, w, nbins, layout, two):
+    frame = torch.zeros((h, w), dtype=torch.uint8, device="cuda")
+    out = torch.empty(ihist.out_shape(h, w, nbins, layout), dtype=torch.int32, device="cuda")
+    with ihist.Batch([frame] * n, nbins, [layout] * n, outs=[out] * n) as batch:
+        assert ihist.two_launch_batch(batch.handle) == two
+
+
+def test_a_frame_of_another_kind_keeps_the_batch_in_two_launches():
+    frame = torch.zeros((1080, 1920), dtype=torch.uint8, device="cuda")
+    out = torch.empty(1080 * 1920 * 32, dtype=torch.int32, device="cuda")
+    for extra in ((PIXEL, 32), (BIN, 256)):
+        frames = [frame] * 40
+        bins, layouts = [8] * 39 + [extra[1]], [BIN] * 39 + [extra[0]]
+        outs = [out[:1080 * 1920 * 8].view(8, 1080, 1920)] * 39 + [
+            torch.empty(ihist.out_shape(1080, 1920, extra[1], extra[0]), dtype=torch.int32, device="cuda")]
+        with ihist.Batch(frames, bins, layouts, outs=outs) as batch:
+            assert ihist.two_launch_batch(batch.handle)
