@@ -262,29 +262,34 @@ int bands_count_class(const BandDesc &f) {
   return (int)std::min<size_t>(4, kSm / (count_smem_bytes(f) + kOther));
 }
 
-// One launch per run of frames of the same kernel, at most kBatchFrames each.
+BandRun bands_run(bool count, int kernel, const BandDesc *d_desc) {
+  BandRun r;
+  r.count = count;
+  r.kernel = kernel;
+  r.threads = count ? (unsigned)kCountThreads : kernel == 5 ? 256u : kernel >= 4 ? 128u : 32u * kSegWarps;
+  r.smem = !count && kernel < 4 ? emit_smem_bytes(kSegWarps, 32) : 0;
+  r.batch.frames = d_desc;
+  r.batch.n = 0;
+  return r;
+}
+
+bool bands_run_add(BandRun *r, const BandDesc &f) {
+  BandBatch &b = r->batch;
+  if (b.n == kBatchFrames) return false;
+  const unsigned int ctas = r->count ? count_ctas(f) : emit_ctas(f, r->kernel);
+  b.end[b.n] = ctas + (b.n > 0 ? b.end[b.n - 1] : 0u);
+  ++b.n;
+  if (r->count || r->kernel >= 4) r->smem = std::max(r->smem, r->count ? count_smem_bytes(f) : emit_smem(f, r->kernel));
+  return true;
+}
+
 int launch_bands_batch(const BandRun *runs, int nruns, void *stream) {
-  for (int i = 0; i < nruns; ++i) {
-    const BandRun &r = runs[i];
-    BandBatch b;
-    b.frames = r.d_desc;
-    b.n = r.n;
-    unsigned int total = 0;
-    size_t smem = 0;
-    for (int j = 0; j < r.n; ++j) {
-      const BandDesc &f = r.h_desc[j];
-      total += r.count ? count_ctas(f) : emit_ctas(f, r.kernel);
-      smem = std::max(smem, r.count ? count_smem_bytes(f) : emit_smem(f, r.kernel));
-      b.end[j] = total;
-    }
-    const unsigned int threads = r.count ? (unsigned)kCountThreads : r.kernel == 5 ? 256u : r.kernel >= 4 ? 128u : 32u * kSegWarps;
-    if (!r.count && r.kernel < 4) smem = emit_smem_bytes(kSegWarps, 32);
-    if (launch(r.count ? count_batch_fn(r.kernel) : emit_batch_fn(r.kernel), total, 1u, 1u, threads, smem, b, stream) !=
-        cudaSuccess) {
+  for (const BandRun *r = runs; r < runs + nruns; ++r)
+    if (launch(r->count ? count_batch_fn(r->kernel) : emit_batch_fn(r->kernel), r->batch.end[r->batch.n - 1], 1u, 1u,
+               r->threads, r->smem, r->batch, stream) != cudaSuccess) {
       cudaGetLastError();
       return IHIST_ERR_CUDA;
     }
-  }
   return IHIST_OK;
 }
 

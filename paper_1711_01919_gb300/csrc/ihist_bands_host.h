@@ -48,14 +48,18 @@ int launch_bands(const BandDesc &f, int mode, int layout, void *stream);
 // Count CTAs per SM that a frame's shared memory allows (1..4).
 int bands_count_class(const BandDesc &f);
 
-// One launch of a batch: n frames (at most kBatchFrames) through the count
-// kernel of a binning or the emit kernel of a kind; their descriptors on the
-// device and on the host.  The launch must find these descriptors on the device.
+// One launch of a batch: at most kBatchFrames frames through the count kernel of
+// a binning or the emit kernel of a kind, whose descriptors the launch must find
+// on the device from d_desc on.
 struct BandRun {
   bool count;
-  int kernel, n;
-  const BandDesc *d_desc, *h_desc;
+  int kernel;
+  unsigned int threads;
+  size_t smem;
+  BandBatch batch;
 };
+BandRun bands_run(bool count, int kernel, const BandDesc *d_desc);
+bool bands_run_add(BandRun *r, const BandDesc &f);  // false: the launch is full
 int launch_bands_batch(const BandRun *runs, int nruns, void *stream);
 
 }  // namespace host

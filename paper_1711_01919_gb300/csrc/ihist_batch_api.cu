@@ -209,24 +209,25 @@ struct ihist_batch_s {
   std::vector<char *> slot_base;
   std::vector<size_t> slot_bytes;
   BandDesc *d_bc, *d_be;               // descriptors by count kernel and by emit kernel
-  std::vector<BandDesc> bc, be;        // the current binding's, in those orders
-  std::vector<BandRun> runs;           // its launches; empty: the look-back kernel
+  std::vector<BandRun> runs;           // the current binding's launches; empty: the look-back kernel
   // Pinned staging of the descriptors, two sets used by alternate bindings:
   // a binding waits only for the copy made from its set two bindings ago,
   // so a caller can bind and launch ahead of the GPU.  h_* point at the set
-  // of the binding being built; staged[i] marks set i's last copy done.
+  // of the binding being built; staged[i] marks set i's last copy done.  A set
+  // holds one array a row, as the device does (kRows), so that a binding is one
+  // 2-D copy of the rows' first n elements: a copy for each array cost a binding
+  // of 2 frames 11.6 us of host time instead of 5.0, of 128 35 instead of 19.
+  size_t row_pitch;
   struct Staging {
-    FrameDesc *fd, *fdq;
-    CUtensorMap *tm;
-    unsigned int *end, *bins_end;
+    char *rows;
     uint32_t *lut;
-    BandDesc *bc, *be;  // behind fd, in its allocation
   } stage_sets[2];
   cudaEvent_t staged[2];
   int stage_cur;
   FrameDesc *h_fd, *h_fdq;
   CUtensorMap *h_tm;
   unsigned int *h_end, *h_bins_end;
+  BandDesc *h_bc, *h_be;
   uint32_t *h_lut;
   cudaEvent_t uploaded;
   // The last launch's completion: `banded` after a launch of the two-launch path
@@ -242,6 +243,11 @@ struct ihist_batch_s {
   void *bound_stream, *banded_stream;
   bool bound_wait, banded_wait;
 };
+
+// The rows of a staging set and of the device's descriptors; the last two only
+// for bindings that take the two-launch path.
+enum { kRowFd, kRowFdq, kRowTm, kRowEnd, kRowBinsEnd, kRowBc, kRowBe, kRows };
+constexpr size_t kRowElem = std::max(std::max(sizeof(FrameDesc), sizeof(BandDesc)), sizeof(CUtensorMap));
 
 // TMA descriptor of the plane the scan reads (the frame, or its joint-bin plane).
 static bool encode_frame_map(const uint8_t *in, size_t pitch, int h, int w, int R, CUtensorMap *map) {
@@ -309,16 +315,17 @@ static bool look_back_faster(const ihist_frame_t *frames, int n) {
   return mp > (2 * wide > px ? 2 * limit : limit);
 }
 
-// Describe the frames for the two-launch path, in launch order; false if one
-// of them does not take it or does not fit its slot.
-static bool bands_bind(ihist_batch_s *b, const ihist_frame_t *frames, const std::vector<FrameDesc> &fd, int n,
-                       std::vector<BandDesc> *bc, std::vector<BandDesc> *be, std::vector<BandRun> *runs) {
-  if (!b->band_ok) return false;
-  if (look_back_faster(frames, n)) return false;
+// Describe the frames for the two-launch path (in the staging set) and its
+// launches; false if a frame does not take it or does not fit its slot.  order:
+// the frames, largest output first, so that every launch ends on small ones.
+static bool bands_bind(ihist_batch_s *b, const ihist_frame_t *frames, const std::vector<FrameDesc> &fd,
+                       const std::vector<int> &order, std::vector<BandRun> *runs) {
+  const int n = (int)order.size();
+  if (!b->band_ok || look_back_faster(frames, n)) return false;
   std::vector<BandDesc> desc(n);
-  std::vector<int> count(n), kind(n), order(n);  // kernels of each frame: binning and CTAs per SM, emit kind
-  int least = 4;                // CTAs per SM of one launch for all
-  unsigned long long ctas = 0;  // and its CTAs
+  std::vector<unsigned char> count(n), kind(n);  // kernels of each frame: binning and CTAs per SM, emit kind
+  int least = 4;                                 // CTAs per SM of one launch for all
+  unsigned long long ctas = 0;                   // and its CTAs
   for (int i = 0; i < n; ++i) {
     const ihist_frame_t &fr = frames[i];
     if (!bands_fit(fr.h, fr.w, fr.layout)) return false;
@@ -347,34 +354,32 @@ static bool bands_bind(ihist_batch_s *b, const ihist_frame_t *frames, const std:
         stride *= f.jmul[c];
       }
     }
-    count[i] = 4 * mode + bands_count_class(f) - 1;
+    count[i] = (unsigned char)(4 * mode + bands_count_class(f) - 1);
     least = std::min(least, count[i] % 4 + 1);
     ctas += count_ctas(f);
-    kind[i] = bands_kind(f, fr.layout);
-    order[i] = i;
+    kind[i] = (unsigned char)bands_kind(f, fr.layout);
   }
   // One launch where it is a few waves at most (7 frames of 640x480 x 16 and
   // one of x 128: 56 us in one, 64 in two).
   if (ctas <= 4ull * least * b->sms)
-    for (int &c : count) c -= c % 4;
-  bc->clear();
-  be->clear();
-  runs->clear();
+    for (unsigned char &c : count) c -= c % 4;
+  constexpr int kKeys = std::max(4 * (kBinJoint + 1), kBandKinds);
   for (int pass = 0; pass < 2; ++pass) {
-    const std::vector<int> &key = pass ? kind : count;
-    std::vector<BandDesc> *to = pass ? be : bc;
-    // by kernel, then largest first, so that a launch ends on small frames
-    std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
-      if (key[a] != key[c]) return key[a] < key[c];
-      return ihist_output_bytes(frames[a].h, frames[a].w, frames[a].nbins) >
-             ihist_output_bytes(frames[c].h, frames[c].w, frames[c].nbins);
-    });
-    for (int i = 0; i < n; ++i) {
-      to->push_back(desc[order[i]]);
-      const int k = key[order[i]];
-      if (i == 0 || k != key[order[i - 1]] || runs->back().n == kBatchFrames)
-        runs->push_back(BandRun{pass == 0, pass ? k : k / 4, 0, (pass ? b->d_be : b->d_bc) + i, nullptr});
-      ++runs->back().n;
+    const std::vector<unsigned char> &key = pass ? kind : count;
+    BandDesc *to = pass ? b->h_be : b->h_bc, *dev = pass ? b->d_be : b->d_bc;
+    int at = 0, held[kKeys] = {};
+    for (int i = 0; i < n; ++i) ++held[key[i]];
+    for (int k = 0; k < kKeys; ++k) {
+      if (!held[k]) continue;
+      runs->push_back(bands_run(pass == 0, pass ? k : k / 4, dev + at));
+      for (int i : order) {
+        if (key[i] != k) continue;
+        if (!bands_run_add(&runs->back(), desc[i])) {
+          runs->push_back(bands_run(pass == 0, pass ? k : k / 4, dev + at));
+          bands_run_add(&runs->back(), desc[i]);
+        }
+        to[at++] = desc[i];
+      }
     }
   }
   return true;
@@ -383,11 +388,15 @@ static bool bands_bind(ihist_batch_s *b, const ihist_frame_t *frames, const std:
 // Point h_* at staging set i.
 static void use_staging(ihist_batch_s *b, int i) {
   b->stage_cur = i;
-  b->h_fd = b->stage_sets[i].fd;
-  b->h_fdq = b->stage_sets[i].fdq;
-  b->h_tm = b->stage_sets[i].tm;
-  b->h_end = b->stage_sets[i].end;
-  b->h_bins_end = b->stage_sets[i].bins_end;
+  char *rows = b->stage_sets[i].rows;
+  auto row = [&](int r) { return rows + r * b->row_pitch; };
+  b->h_fd = reinterpret_cast<FrameDesc *>(row(kRowFd));
+  b->h_fdq = reinterpret_cast<FrameDesc *>(row(kRowFdq));
+  b->h_tm = reinterpret_cast<CUtensorMap *>(row(kRowTm));
+  b->h_end = reinterpret_cast<unsigned int *>(row(kRowEnd));
+  b->h_bins_end = reinterpret_cast<unsigned int *>(row(kRowBinsEnd));
+  b->h_bc = reinterpret_cast<BandDesc *>(row(kRowBc));
+  b->h_be = reinterpret_cast<BandDesc *>(row(kRowBe));
   b->h_lut = b->stage_sets[i].lut;
 }
 
@@ -438,11 +447,12 @@ static int batch_bind(ihist_batch_s *b, const ihist_frame_t *frames, int n) {
   // bins: 5.235 -> 5.142 ms against the caller's order).  Each frame's descriptor carries its own slot's
   // carries, table and plane, so only the order of the items changes.
   std::vector<int> order(n);
-  for (int i = 0; i < n; ++i) order[i] = i;
-  std::stable_sort(order.begin(), order.end(), [&](int a, int c) {
-    return ihist_output_bytes(frames[a].h, frames[a].w, frames[a].nbins) >
-           ihist_output_bytes(frames[c].h, frames[c].w, frames[c].nbins);
-  });
+  std::vector<size_t> bytes(n);
+  for (int i = 0; i < n; ++i) {
+    order[i] = i;
+    bytes[i] = ihist_output_bytes(frames[i].h, frames[i].w, frames[i].nbins);
+  }
+  std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return bytes[a] > bytes[c]; });
   unsigned long long brun = 0;
   for (int i = 0; i < n; ++i) {
     brun += (unsigned long long)frames[i].nbins;
@@ -466,18 +476,9 @@ static int batch_bind(ihist_batch_s *b, const ihist_frame_t *frames, int n) {
     b->h_end[k] = (unsigned int)run;
     b->h_fd[k] = fd[i];
   }
-  std::vector<BandDesc> bc, be;
   std::vector<BandRun> runs;
-  if (bands_bind(b, frames, fd, n, &bc, &be, &runs)) {
-    std::memcpy(b->stage_sets[b->stage_cur].bc, bc.data(), (size_t)n * sizeof(BandDesc));
-    std::memcpy(b->stage_sets[b->stage_cur].be, be.data(), (size_t)n * sizeof(BandDesc));
-  } else {
-    runs.clear();
-  }
-  b->bc.swap(bc);
-  b->be.swap(be);
+  if (!bands_bind(b, frames, fd, order, &runs)) runs.clear();
   b->runs.swap(runs);
-  for (BandRun &r : b->runs) r.h_desc = r.count ? b->bc.data() + (r.d_desc - b->d_bc) : b->be.data() + (r.d_desc - b->d_be);
   b->fd.assign(fd.begin(), fd.end());
   b->io.assign(frames, frames + n);
   b->n = n;
@@ -489,20 +490,12 @@ static int batch_bind(ihist_batch_s *b, const ihist_frame_t *frames, int n) {
 }
 
 static int batch_upload(ihist_batch_s *b, cudaStream_t s) {
-  const int n = b->n;
-  if (cudaMemcpyAsync(b->d_fd, b->h_fd, (size_t)n * sizeof(FrameDesc), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemcpyAsync(b->d_fdq, b->h_fdq, (size_t)n * sizeof(FrameDesc), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemcpyAsync(b->d_tm, b->h_tm, (size_t)n * sizeof(CUtensorMap), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemcpyAsync(b->d_end, b->h_end, (size_t)n * sizeof(unsigned int), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemcpyAsync(b->d_bins_end, b->h_bins_end, (size_t)n * sizeof(unsigned int), cudaMemcpyHostToDevice, s) !=
-          cudaSuccess ||
-      (b->lut && cudaMemcpyAsync(b->d_lut, b->h_lut, (size_t)n * 256 * sizeof(uint32_t), cudaMemcpyHostToDevice,
-                                 s) != cudaSuccess) ||
-      (!b->runs.empty() &&
-       (cudaMemcpyAsync(b->d_bc, b->stage_sets[b->stage_cur].bc, (size_t)n * sizeof(BandDesc), cudaMemcpyHostToDevice,
-                        s) != cudaSuccess ||
-        cudaMemcpyAsync(b->d_be, b->stage_sets[b->stage_cur].be, (size_t)n * sizeof(BandDesc), cudaMemcpyHostToDevice,
-                        s) != cudaSuccess)) ||
+  const size_t n = (size_t)b->n;
+  const ihist_batch_s::Staging &st = b->stage_sets[b->stage_cur];
+  if (cudaMemcpy2DAsync(b->d_fd, b->row_pitch, st.rows, b->row_pitch, n * kRowElem, b->runs.empty() ? kRowBc : kRows,
+                        cudaMemcpyHostToDevice, s) != cudaSuccess ||
+      (b->lut && cudaMemcpyAsync(b->d_lut, b->h_lut, n * 256 * sizeof(uint32_t), cudaMemcpyHostToDevice, s) !=
+                     cudaSuccess) ||
       cudaEventRecord(b->staged[b->stage_cur], s) != cudaSuccess)
     return IHIST_ERR_CUDA;
   return IHIST_OK;
@@ -522,11 +515,7 @@ extern "C" void ihist_batch_destroy(ihist_batch_t b) {
   if (b->banded) cudaEventDestroy(b->banded);
   for (int i = 0; i < 2; ++i) {
     ihist_batch_s::Staging &st = b->stage_sets[i];
-    if (st.fd) cudaFreeHost(st.fd);
-    if (st.fdq) cudaFreeHost(st.fdq);
-    if (st.tm) cudaFreeHost(st.tm);
-    if (st.end) cudaFreeHost(st.end);
-    if (st.bins_end) cudaFreeHost(st.bins_end);
+    if (st.rows) cudaFreeHost(st.rows);
     if (st.lut) cudaFreeHost(st.lut);
   }
   if (b->ws) cudaFree(b->ws);
@@ -746,20 +735,9 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
   const size_t o_flags = off;
   off = align_up(off + nci_total * sizeof(uint32_t), 256);
   const size_t zero_end = off;
-  const size_t o_fd = off;
-  off = align_up(off + (size_t)n * sizeof(FrameDesc), 256);
-  const size_t o_fdq = off;
-  off = align_up(off + (size_t)n * sizeof(FrameDesc), 256);
-  const size_t o_tm = off;
-  off = align_up(off + (size_t)n * sizeof(CUtensorMap), 256);
-  const size_t o_bc = off;
-  off = align_up(off + (size_t)n * sizeof(BandDesc), 256);
-  const size_t o_be = off;
-  off = align_up(off + (size_t)n * sizeof(BandDesc), 256);
-  const size_t o_end = off;
-  off = align_up(off + (size_t)n * sizeof(unsigned int), 256);
-  const size_t o_bend = off;
-  off = align_up(off + (size_t)n * sizeof(unsigned int), 256);
+  const size_t o_rows = off;
+  b->row_pitch = align_up((size_t)n * kRowElem, 256);
+  off += kRows * b->row_pitch;
   const size_t o_lut = off;
   if (lut) off = align_up(off + (size_t)n * 256 * sizeof(uint32_t), 256);
   const size_t o_carry = off;
@@ -783,17 +761,10 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
       [&]() {
         for (int i = 0; i < 2; ++i) {
           ihist_batch_s::Staging &st = b->stage_sets[i];
-          if (cudaMallocHost((void **)&st.fd, (size_t)n * (sizeof(FrameDesc) + 2 * sizeof(BandDesc))) != cudaSuccess ||
-              cudaMallocHost((void **)&st.fdq, (size_t)n * sizeof(FrameDesc)) != cudaSuccess ||
-              cudaMallocHost((void **)&st.tm, (size_t)n * sizeof(CUtensorMap)) != cudaSuccess ||
-              cudaMallocHost((void **)&st.end, (size_t)n * sizeof(unsigned int)) != cudaSuccess ||
-              cudaMallocHost((void **)&st.bins_end, (size_t)n * sizeof(unsigned int)) != cudaSuccess ||
+          if (cudaMallocHost((void **)&st.rows, kRows * b->row_pitch) != cudaSuccess ||
               (lut && cudaMallocHost((void **)&st.lut, (size_t)n * 256 * sizeof(uint32_t)) != cudaSuccess) ||
               cudaEventCreateWithFlags(&b->staged[i], cudaEventDisableTiming) != cudaSuccess)
             return false;
-          static_assert(sizeof(FrameDesc) % alignof(BandDesc) == 0, "bc follows fd");
-          st.bc = reinterpret_cast<BandDesc *>(st.fd + n);
-          st.be = st.bc + n;
         }
         return true;
       }() == false ||
@@ -806,13 +777,14 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
   }
   char *base = static_cast<char *>(b->ws);
   b->ctrl = reinterpret_cast<Ctrl *>(base + o_ctrl);
-  b->d_fd = reinterpret_cast<FrameDesc *>(base + o_fd);
-  b->d_fdq = reinterpret_cast<FrameDesc *>(base + o_fdq);
-  b->d_tm = reinterpret_cast<CUtensorMap *>(base + o_tm);
-  b->d_bc = reinterpret_cast<BandDesc *>(base + o_bc);
-  b->d_be = reinterpret_cast<BandDesc *>(base + o_be);
-  b->d_end = reinterpret_cast<unsigned int *>(base + o_end);
-  b->d_bins_end = reinterpret_cast<unsigned int *>(base + o_bend);
+  auto row = [&](int r) { return base + o_rows + r * b->row_pitch; };
+  b->d_fd = reinterpret_cast<FrameDesc *>(row(kRowFd));
+  b->d_fdq = reinterpret_cast<FrameDesc *>(row(kRowFdq));
+  b->d_tm = reinterpret_cast<CUtensorMap *>(row(kRowTm));
+  b->d_end = reinterpret_cast<unsigned int *>(row(kRowEnd));
+  b->d_bins_end = reinterpret_cast<unsigned int *>(row(kRowBinsEnd));
+  b->d_bc = reinterpret_cast<BandDesc *>(row(kRowBc));
+  b->d_be = reinterpret_cast<BandDesc *>(row(kRowBe));
   if (lut) b->d_lut = reinterpret_cast<uint32_t *>(base + o_lut);
   size_t fo = o_flags, co = o_carry;
   for (int i = 0; i < n; ++i) {
