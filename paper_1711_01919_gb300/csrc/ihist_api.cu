@@ -389,50 +389,50 @@ static int plan_create(int h, int w, int nbins, int layout, const ihist_tune_t *
   const int mode = table ? kBinTable : joint ? kBinJoint : kBinUniform;
   if (banded && table && nbins > 252)  // no byte left for "no bin"
     for (int v = 0; v < 256; ++v) banded = banded && bin_map[v] >= 0;
-  if (banded) {
-    const int brc = bands_prepare(mode, layout);
-    if (brc != IHIST_OK) {
-      delete p;
-      return brc;
-    }
-  }
-  p->banded = banded;
+  banded = banded && bands_prepare(mode, layout) == IHIST_OK;
 
   // workspace: control blocks, then the two-launch path's counts or the
   // look-back kernel's flags, column-count aggregates, left counts and
   // inclusive rows
-  const size_t nci = banded ? 0 : (size_t)p->nbands * p->ngroups * p->nchunks;
-  size_t off = 0;
-  const size_t o_ctrl = off;
-  off = align_up(off + sizeof(Ctrl), 256);
-  const size_t o_ctrl_alt = off;
-  off = align_up(off + sizeof(Ctrl), 256);
-  const size_t o_flags = off;
-  off = align_up(off + nci * sizeof(uint32_t), 256);
-  const size_t nhs = !banded && nsegs > 1 ? (size_t)p->nbands * p->ngroups * nsegs : 0;  // segment records
-  const size_t o_hflags = off;
-  off = align_up(off + nhs * sizeof(uint32_t), 256);
-  const size_t o_cnt = off;
-  off = align_up(off + nci * kChunk * (p->G / 4) * sizeof(uint32_t), 256);
-  const size_t o_left = off;
-  off = align_up(off + nci * p->G * sizeof(uint32_t), 256);
-  const size_t o_incl = off;
-  off = align_up(off + nci * p->G * kChunk * sizeof(uint32_t), 256);
-  const size_t o_hagg = off;
-  off = align_up(off + nhs * ((size_t)p->R * p->G + p->G) * sizeof(uint32_t), 256);
-  const size_t o_lut = off;
-  if (table) off = align_up(off + 256 * sizeof(uint32_t), 256);
-  const size_t o_idx = off;
+  size_t o_ctrl, o_ctrl_alt, o_flags, o_hflags, o_cnt, o_left, o_incl, o_hagg, o_lut, o_idx, o_band, nhs;
   p->idx_pitch = align_up((size_t)w, 16);
-  if (joint && !banded) off = align_up(off + (size_t)h * p->idx_pitch, 256);
-  const size_t o_band = off;
-  if (banded) off += bands_layout(&band, nullptr);
-  p->ws_bytes = off;
-  if (cudaMalloc(&p->ws, p->ws_bytes) != cudaSuccess) {
+  auto layout_ws = [&]() {
+    const size_t nci = banded ? 0 : (size_t)p->nbands * p->ngroups * p->nchunks;
+    nhs = !banded && nsegs > 1 ? (size_t)p->nbands * p->ngroups * nsegs : 0;  // segment records
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+      const size_t at = off;
+      off = align_up(off + bytes, 256);
+      return at;
+    };
+    o_ctrl = take(sizeof(Ctrl));
+    o_ctrl_alt = take(sizeof(Ctrl));
+    o_flags = take(nci * sizeof(uint32_t));
+    o_hflags = take(nhs * sizeof(uint32_t));
+    o_cnt = take(nci * kChunk * (p->G / 4) * sizeof(uint32_t));
+    o_left = take(nci * p->G * sizeof(uint32_t));
+    o_incl = take(nci * p->G * kChunk * sizeof(uint32_t));
+    o_hagg = take(nhs * ((size_t)p->R * p->G + p->G) * sizeof(uint32_t));
+    o_lut = take(table ? 256 * sizeof(uint32_t) : 0);
+    o_idx = take(joint && !banded ? (size_t)h * p->idx_pitch : 0);
+    o_band = take(banded ? bands_layout(&band, nullptr) : 0);
+    p->ws_bytes = off;
+    return cudaMalloc(&p->ws, p->ws_bytes) == cudaSuccess;
+  };
+  bool got = layout_ws();
+  if (!got && banded) {
+    // the look-back kernel's carries may still fit (few bins: 3840x2160 x 4
+    // takes 9.9 MB of counts or 3.6 MB of carries)
+    cudaGetLastError();
+    banded = false;
+    got = layout_ws();
+  }
+  if (!got) {
     cudaGetLastError();
     delete p;
     return IHIST_ERR_OOM;
   }
+  p->banded = banded;
   char *base = static_cast<char *>(p->ws);
   p->ctrl = reinterpret_cast<Ctrl *>(base + o_ctrl);
   p->ctrl_alt = reinterpret_cast<Ctrl *>(base + o_ctrl_alt);

@@ -741,23 +741,35 @@ extern "C" int ihist_batch_plan(const ihist_frame_t *frames, int n, const ihist_
   const size_t o_lut = off;
   if (lut) off = align_up(off + (size_t)n * 256 * sizeof(uint32_t), 256);
   const size_t o_carry = off;
-  for (int i = 0; i < n; ++i) {
-    const size_t nci = b->slot_nci[i];
-    const size_t at = off;
-    off = align_up(off + nci * kChunk * (b->G / 4) * 4, 256);
-    off = align_up(off + nci * b->G * 4, 256);
-    off = align_up(off + nci * b->G * kChunk * 4, 256);
-    off = align_up(off + b->slot_hwords[i] * 4, 256);
-    off = std::max(off, at + band_bytes[i]);
-    b->slot_bytes.push_back(off - at);
+  for (int i = 0; i < n; ++i) b->slot_idx_cap.push_back(idx_bytes_of(frames[i]));
+  size_t o_idx = 0;  // joint-bin planes of the slots planned with joint frames
+  auto allocate = [&]() {
+    off = o_carry;
+    b->slot_bytes.clear();
+    for (int i = 0; i < n; ++i) {
+      const size_t nci = b->slot_nci[i];
+      const size_t at = off;
+      off = align_up(off + nci * kChunk * (b->G / 4) * 4, 256);
+      off = align_up(off + nci * b->G * 4, 256);
+      off = align_up(off + nci * b->G * kChunk * 4, 256);
+      off = align_up(off + b->slot_hwords[i] * 4, 256);
+      if (b->band_ok) off = std::max(off, at + band_bytes[i]);
+      b->slot_bytes.push_back(off - at);
+    }
+    o_idx = off;
+    for (int i = 0; i < n; ++i) off = align_up(off + b->slot_idx_cap[i], 256);
+    b->ws_bytes = off;
+    return cudaMalloc(&b->ws, b->ws_bytes) == cudaSuccess;
+  };
+  bool got = allocate();
+  if (!got && b->band_ok) {
+    // the look-back kernel's carries may still fit (64 frames of 1920x1080 x 4:
+    // 172 MB with room for counts, 57 without)
+    cudaGetLastError();
+    b->band_ok = false;
+    got = allocate();
   }
-  const size_t o_idx = off;  // joint-bin planes of the slots planned with joint frames
-  for (int i = 0; i < n; ++i) {
-    b->slot_idx_cap.push_back(idx_bytes_of(frames[i]));
-    off = align_up(off + b->slot_idx_cap[i], 256);
-  }
-  b->ws_bytes = off;
-  if (cudaMalloc(&b->ws, b->ws_bytes) != cudaSuccess ||
+  if (!got ||
       [&]() {
         for (int i = 0; i < 2; ++i) {
           ihist_batch_s::Staging &st = b->stage_sets[i];
