@@ -166,9 +166,12 @@ static bool look_back_faster(const BandDesc &f, int layout, bool table) {
     // records of one or two whole sectors, which that kernel stores complete:
     // 4320x7680 x 8 440 us against 460 here, 400x65532 x 8 and x 16 1.16x and
     // 1.07x faster (x 12 0.8x; here a CTA also adds up the counts of all chunks
-    // to its left), 4320x5800 x 8 0.94x
-    return (f.B == 8 && px > (f.W > 48000 ? 16000000 : 30000000)) ||
+    // to its left), 4320x5800 x 8 0.94x, 600x65535 x 8 (rows off 16 bytes) 0.97x
+    return (f.B == 8 && f.W % 4 == 0 && px > (f.W > 48000 ? 16000000 : 30000000)) ||
            (f.B == 16 && f.W > 62000 && px > 24000000);
+  // Four bins only, counted in a pass as long as their stores: 4800x8192 x 4 168
+  // us here, 161 there, 7680x4320 x 4 0.93x.
+  if (layout == IHIST_QUAD_MAJOR && f.B == 4 && f.W % 16 == 0 && px > 38000000) return true;
   // Bins and counts that L2 does not hold, where its own loads are whole (rows
   // of 16-byte multiples): bin-major 3840x2160 x 128 (58 MB) 660 us here, 663
   // there, x 192 (83 MB) 998 / 967, 3200x2500 x 160 (68 MB) 788 / 808, 4000x3000

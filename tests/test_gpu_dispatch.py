@@ -33,6 +33,7 @@ def _lib():
     (4320, 7680, 256, PIXEL, True),
     # whole small records of large pixel-major frames
     (4320, 7680, 8, PIXEL, False), (4320, 7680, 6, PIXEL, True), (3000, 4000, 8, PIXEL, True),
+    (600, 65532, 8, PIXEL, False), (600, 65535, 8, PIXEL, True), (8192, 4800, 4, QUAD, False), (4320, 7680, 4, QUAD, True),
     (400, 65532, 16, PIXEL, False), (400, 65532, 12, PIXEL, True), (600, 30000, 16, PIXEL, True),
 ])
 def test_plans(h, w, nbins, layout, two):
