@@ -347,7 +347,7 @@ def run_mp64_slice(args) -> int:
         if plan.status() != ihist.IHIST_OK:
             raise SystemExit("device status error in the 8192-column slice")
         ms = [ev[2 * k].elapsed_time(ev[2 * k + 1]) for k in range(args.warmup, args.warmup + args.steps)]
-        print(json.dumps({"case": "mp64-slice", "rows": h, "W": w, "B": b, "tile": plan.tune,
+        print(json.dumps({"case": "mp64-slice", "rows": h, "W": w, "B": b, "tile": tile_of(plan),
                           "full_frame_tile": tune, "launch_ms": ms,
                           "bytes_per_launch": h * w * b * 4 + h * w}), flush=True)
     return 0
@@ -533,12 +533,18 @@ def _median_ms(fn, stream, reps: int = 50, warm: int = 10) -> float:
     return _time_ms(fn, stream, reps, warm)["median"]
 
 
+def tile_of(plan):
+    """The tiling a plan's frames run with, or the path that has none."""
+    from paper_1711_01919_gb300 import ihist
+    return "two launches (count, emit)" if ihist.two_launch_plan(plan.handle) else plan.tune
+
+
 def configs_report(stream, peak: float) -> dict:
     """The other workloads of the method, each timed on its own (median and
     min of 50 after 10 warm-ups, CUDA events): one 640x480 frame with 32 bins and 1000
     queries per launch pair (8 frames and 8 outputs in rotation, 315 MB > L2);
-    a 256-frame batch of uneven size (320x240 .. 1920x1080, 16/32/64 bins) in
-    one persistent launch, default and autotuned tiling, the autotuned one
+    a 256-frame batch of uneven size (320x240 .. 1920x1080, 16/32/64 bins),
+    default and autotuned (as live launches), the autotuned one
     also replayed from a captured CUDA graph; one 8192x8192 frame with 128
     bins (34.4 GB out) and 2^20 queries on it."""
     import torch
@@ -573,7 +579,7 @@ def configs_report(stream, peak: float) -> dict:
                           "us_per_frame_min": tm["min"] * 1e3 / 64,
                           "gbs": byts / ms / 1e6, "frac": byts / ms / 1e6 / peak,
                           "form": "ihist_compute + ihist_query per frame" + (", overlap=1" if tune else ""),
-                          "tile": plan.tune}
+                          "tile": tile_of(plan)}
     del fr, ou, rects, q
     # 256 uneven frames in one launch
     specs = synth.uneven_batch_specs(synth.workload_seed(3), 256)
@@ -585,7 +591,7 @@ def configs_report(stream, peak: float) -> dict:
     ou = [torch.empty((nb, h, w), dtype=torch.int32, device="cuda") for (h, w, nb, sd) in specs]
     nbs = [nb for (h, w, nb, sd) in specs]
     byts = sum(h * w * nb * 4 + h * w for (h, w, nb, sd) in specs)
-    entry = {"frames": 256, "algorithmic_bytes": byts, "form": "one ihist_batch_compute launch"}
+    entry = {"frames": 256, "algorithmic_bytes": byts, "form": "one ihist_batch_compute"}
     # the autotuner picks the layout (no queries in this workload) and, for
     # it, the launch shape
     auto_layout, auto_tune, layout_ms = autotune.tune_batch_layout([(h, w, nb) for (h, w, nb, sd) in specs], 0)
@@ -597,11 +603,12 @@ def configs_report(stream, peak: float) -> dict:
             if batch.status() != ihist.IHIST_OK:
                 raise SystemExit("device status error in the uneven batch")
             entry[label] = {"ms": ms, "ms_min": tm["min"], "frames_per_s": 256e3 / ms, "gbs": byts / ms / 1e6,
-                            "frac": byts / ms / 1e6 / peak, "items": batch.items(), "layout": names[layout]}
+                            "frac": byts / ms / 1e6 / peak, "items": batch.items(), "layout": names[layout],
+                            "path": "two-launch" if ihist.two_launch_batch(batch.handle) else "look-back"}
             if label == "autotuned":
                 entry[label]["tune"] = auto_tune
                 entry[label]["layout_ms_while_tuning"] = {names[k]: v for k, v in layout_ms.items()}
-                # the same launch captured once in a CUDA graph and replayed
+                # captured once in a CUDA graph and replayed (the look-back kernel with that tiling)
                 g = torch.cuda.CUDAGraph()
                 with torch.cuda.graph(g):
                     batch.compute()
@@ -655,7 +662,7 @@ def configs_report(stream, peak: float) -> dict:
                                       "clocks": clk, "query_ms_2p20_rects": qms, "query_ms_min": tq["min"],
                                       "query_sorted_ms_2p20_rects": {"bins_per_pass_%d" % k: v
                                                                      for k, v in sorted_ms.items()},
-                                      "tile": plan.tune}
+                                      "tile": tile_of(plan)}
         rep["mp64_8192x8192_b128"].update(query_gather_report(out, qms, 1 << 20, b, stream))
     del img, out, rects, q
     torch.cuda.empty_cache()
@@ -690,8 +697,8 @@ def query_gather_report(hist, query_ms: float, nrects: int, nbins: int, stream) 
 
 def mappings_report(stream, peak: float) -> dict:
     """The paper's GPU mappings (CW-STS, CW-TiS, WF-TiS; comparison kernels
-    built on this GPU) against the fused look-back kernel, one 1080p frame
-    with 64 bins each, same output, same algorithmic bytes."""
+    built on this GPU) against the default plan and the fused look-back kernel,
+    one 1080p frame with 64 bins each, same output, same algorithmic bytes."""
     import torch
 
     from paper_1711_01919_gb300 import ihist, synth
@@ -707,14 +714,14 @@ def mappings_report(stream, peak: float) -> dict:
                                                             work.data_ptr() if nb else 0, s), stream)
         rep[name] = {"ms_per_frame": ms, "frames_per_s": 1e3 / ms, "frac": byts / ms / 1e6 / peak}
         del work
-    with ihist.Plan(H, W, NBINS) as plan:
-        ms = _median_ms(lambda: ihist.ihist_compute(plan.handle, img.data_ptr(), W, out.data_ptr(), s), stream)
-    rep["fused_look_back"] = {"ms_per_frame": ms, "frames_per_s": 1e3 / ms, "frac": byts / ms / 1e6 / peak}
-    # the same frame into the pixel-major layout [y][x][b]
-    with ihist.Plan(H, W, NBINS, ihist.IHIST_PIXEL_MAJOR) as plan:
-        ms = _median_ms(lambda: ihist.ihist_compute(plan.handle, img.data_ptr(), W, out.data_ptr(), s), stream)
-        rep["fused_look_back_pixel_major"] = {"ms_per_frame": ms, "frames_per_s": 1e3 / ms,
-                                              "frac": byts / ms / 1e6 / peak, "tile": plan.tune}
+    # the default plan, and the fused look-back kernel at its default tiling;
+    # then the same frame into the pixel-major layout [y][x][b]
+    for suffix, layout in (("", ihist.IHIST_BIN_MAJOR), ("_pixel_major", ihist.IHIST_PIXEL_MAJOR)):
+        for name, tune in (("default_plan", None), ("fused_look_back", {"ctas_per_sm": 32})):
+            with ihist.Plan(H, W, NBINS, layout, tune=tune) as plan:
+                ms = _median_ms(lambda: ihist.ihist_compute(plan.handle, img.data_ptr(), W, out.data_ptr(), s), stream)
+                rep[name + suffix] = {"ms_per_frame": ms, "frames_per_s": 1e3 / ms, "frac": byts / ms / 1e6 / peak,
+                                      "tile": tile_of(plan)}
     return rep
 
 
@@ -853,7 +860,7 @@ def other_bins_report(d_frames, outs, stream, steps: int = 5) -> dict:
         sec = a.elapsed_time(b) / 1000.0
         byts = steps * n * (H * W * NBINS * 4 + read_bytes)
         out[name] = {"frames_per_s": steps * n / sec, "gbs": byts / sec / 1e9,
-                     "form": "%d x ihist_compute per step" % n, "tile": plan.tune}
+                     "form": "%d x ihist_compute per step" % n, "tile": tile_of(plan)}
         plan.close()
     # the same frames in one batched launch each: the edges as value -> bin
     # tables, and the joint RGB bins (joint-bin planes, then one scan launch)
@@ -1138,7 +1145,7 @@ def main():
                 "plain_per_frame": {
                     "value": job_throughput(NFRAMES, pf_steps, world, plain_ms), "unit": "frames/s",
                     "steps": pf_steps, "form": "%d x (ihist_compute + ihist_query) per step" % NFRAMES,
-                    "tile": plan.tune},
+                    "tile": tile_of(plan)},
                 "plain_per_frame_overlapped": {
                     "value": job_throughput(NFRAMES, pf_steps, world, overlap_ms), "unit": "frames/s",
                     "steps": pf_steps, "form": "as plain_per_frame, plan tune overlap=1 (programmatic "
