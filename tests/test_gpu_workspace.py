@@ -1,6 +1,8 @@
 """Plans and batches made while the device has room for the look-back kernel's
 carries but not for the two-launch path's counts: they are made all the same,
 and take the look-back kernel."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -12,7 +14,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 TILED = {"ctas_per_sm": 32}
-BLOCK = 2 << 20  # device memory is handed out in pieces of this size
+PIECE = 2 << 20  # device memory is handed out in pieces of this size
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -24,17 +26,31 @@ def _lib():
         pytest.skip("no CUDA device")
 
 
-def fill_device(leave):
-    """Allocate all but about `leave` bytes of the device, in large pieces then small ones."""
-    held = []
-    torch.cuda.empty_cache()
-    for piece in (8 << 30, 512 << 20, 64 << 20, BLOCK):
-        while torch.cuda.mem_get_info()[0] > leave + 2 * piece:
-            try:
-                held.append(torch.empty(piece, dtype=torch.uint8, device="cuda"))
-            except torch.OutOfMemoryError:
-                break
-    return held
+class Full:
+    """All of the device allocated but `hole` bytes in one piece, past torch's
+    allocator (whose cached blocks would blur the line)."""
+
+    def __init__(self, hole):
+        self.driver, self.held = ctypes.CDLL("libcuda.so.1"), []
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        free = self.take(hole)
+        assert free
+        for piece in (8 << 30, 512 << 20, 64 << 20, PIECE):
+            while True:
+                p = self.take(piece)
+                if not p:
+                    break
+                self.held.append(p)
+        self.driver.cuMemFree_v2(ctypes.c_uint64(free))
+
+    def take(self, n):
+        p = ctypes.c_uint64()
+        return p.value if self.driver.cuMemAlloc_v2(ctypes.byref(p), ctypes.c_size_t(n)) == 0 else 0
+
+    def close(self):
+        for p in self.held:
+            self.driver.cuMemFree_v2(ctypes.c_uint64(p))
 
 
 @pytest.mark.parametrize("kind", ["plan", "batch"])
@@ -58,14 +74,14 @@ def test_made_with_the_look_back_kernels_workspace(kind):
     with make() as a, make(TILED) as b:
         assert two(a.handle) and not two(b.handle)
         counts, carries = nbytes(a), nbytes(b)
-    assert counts > carries + 6 * BLOCK
-    held = fill_device((counts + carries) // 2)
+    hole = carries + PIECE
+    assert counts > hole + 2 * PIECE
+    full = Full(hole)
     try:
         x = make()
         assert nbytes(x) < counts and not two(x.handle)
     finally:
-        held.clear()
-        torch.cuda.empty_cache()
+        full.close()
     with x:
         got = (x.compute(frame, out) if kind == "plan" else x.compute()[0]).cpu().numpy().view(np.uint32)
         assert x.status() == ihist.IHIST_OK
