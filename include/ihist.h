@@ -73,8 +73,11 @@ typedef struct ihist_plan_s *ihist_plan_t;
  * default for the frame shape.  A plan that leaves every tiling field zero
  * (rows_per_band, bins_per_cta, chunks_per_warp, groups_per_cta, ctas_per_sm,
  * warps_per_cta) may take the two-launch path instead (a count kernel, then
- * an emit kernel; bin-major frames up to 12 megapixels, others up to 40),
- * which has no tiling of its own: ihist_plan_get_tune then reports the tiling
+ * an emit kernel): frames of at most 8192 rows, bin-major up to 12 megapixels,
+ * others up to 40, but for those that the fused kernel does faster (many bins
+ * on large frames, whole 32- or 64-byte records of very large pixel-major
+ * ones) and where the device has no room for its workspace.  It has no tiling
+ * of its own: ihist_plan_get_tune then reports the tiling
  * of the fused kernel for the shape, and passing it back selects that kernel.
  * Results are the same words either way.
  *   rows_per_band   R, rows one CTA owns (1..255)
@@ -124,8 +127,8 @@ typedef struct ihist_plan_s *ihist_plan_t;
  *                   kernel in between makes it safe again).  1080p x 64 per
  *                   frame with 1000 queries: 96 us with the default, 94 with
  *                   1; 640x480 x 32 the same: 15.7 and 14.4 us.  Joint plans treat 1 as 0
- *                   (their scan reads the joint-bin plane the kernel before
- *                   it writes); ihist_sequence_host always uses 1 (its
+ *                   (on the fused kernel their scan reads the joint-bin plane
+ *                   that the kernel before it writes); ihist_sequence_host always uses 1 (its
  *                   frames arrive by copy).  Batches ignore it.
  *   reserved        0; ihist_plan_get_tune and ihist_batch_get_tune report 1
  *                   there if the plan, or the batch with its current binding,
@@ -198,10 +201,11 @@ int ihist_edges_table(int nbins, const int *edges, int *bin_of_value);
  * k = (...(q_0 * B_1 + q_1) * B_2 + ...) + q_{C-1}   (channel 0 most
  * significant), so the plan has nbins = prod B_c planes, at most 256
  * (IHIST_ERR_UNSUPPORTED above that or when w * channels > 65535).
- * bins_per_channel is a HOST array of `channels` ints in 1..256.  Each
- * ihist_compute first writes the pixels' joint bins into a plane the plan
- * owns (h x w bytes, one extra read of the frame), then runs the scan on it;
- * the output is H[k][y][x] (or pixel-major) exactly as for nbins uniform
+ * bins_per_channel is a HOST array of `channels` ints in 1..256.  The
+ * two-launch path's count kernel forms the joint bins itself; with the fused
+ * kernel each ihist_compute first writes them into a plane the plan
+ * owns (h x w bytes, one extra read of the frame), then runs the scan on it.
+ * The output is H[k][y][x] (or pixel-major) exactly as for nbins uniform
  * bins.  ihist_query and ihist_sequence_host (frames of h * w * channels
  * bytes) work unchanged. */
 int ihist_plan_joint(int h, int w, int channels, const int *bins_per_channel, int layout,
@@ -214,7 +218,8 @@ int ihist_plan_channels(ihist_plan_t plan);
 /* The tiling a plan resolved to (all fields filled). */
 int ihist_plan_get_tune(ihist_plan_t plan, ihist_tune_t *out);
 
-/* Device workspace bytes the plan holds (carry vectors, flags, control). */
+/* Device workspace bytes the plan holds (carry vectors and flags or the
+ * two-launch path's counts, control). */
 size_t ihist_workspace_bytes(ihist_plan_t plan);
 
 /* Bytes of one integral histogram: h * w * nbins * 4. */
@@ -343,15 +348,23 @@ int ihist_sequence_host(ihist_plan_t plan, const uint8_t *h_frames, size_t frame
                         const int32_t *d_rects, int nrects, uint32_t *d_query,
                         uint32_t *h_query_out, void *stream, void *copy_stream);
 
-/* ---- Batches: many frames of uneven size in one persistent launch -------
+/* ---- Batches: many frames of uneven size in one persistent launch, or two
  *
  * A batch is a work-list over several frames (any mix of shapes, bin counts
  * and layouts): one launch computes every frame's integral histogram, so the
  * ramp and tail of a launch are paid once per batch instead of once per
- * frame.  The same fused kernel runs on each frame (Eq. 1; Sec. 4.4's image
- * sequences as one launch), and results equal ihist_compute's word for word.
- * The launch needs no host-side reset between calls, so it can be captured
- * in a CUDA graph and replayed. */
+ * frame (Eq. 1; Sec. 4.4's image sequences as one launch), and results equal
+ * ihist_compute's word for word.  That launch runs the fused look-back kernel
+ * on each frame.  A batch planned without a tiling, whose frames all fit the
+ * two-launch path (see ihist_tune_t), runs that path's kernels instead, where
+ * they are faster (not with large aligned bin-major batches, nor with many
+ * pixels of few bins): a count launch per binning and size of bin count, then
+ * an emit launch per layout and alignment, each for up to 256 frames.
+ * No call needs a host-side reset before the next, so a batch can be captured
+ * in a CUDA graph and replayed: a captured launch is always the fused
+ * kernel's, which reads the binding on the device and so follows later
+ * bindings.  A joint-bin frame's plane is then made from the frame that was
+ * bound at the capture. */
 typedef struct ihist_batch_s *ihist_batch_t;
 
 /* One frame of a batch.  d_in: h rows of w bytes, row stride in_pitch;
@@ -365,9 +378,9 @@ typedef struct ihist_batch_s *ihist_batch_t;
  * for ihist_plan_joint: d_in holds `channels` interleaved bytes per pixel
  * (in_pitch >= w * channels), channel c is cut into bins_per_channel[c]
  * uniform bins (channel 0 the most significant digit) and nbins must equal
- * their product; bin_of_value must then be NULL.  The batch computes each
- * joint frame's joint-bin plane (one byte per pixel, in its workspace) just
- * before the scan.  A zero-initialised struct is a uniform one-channel
+ * their product; bin_of_value must then be NULL.  Before the fused kernel's
+ * launch the batch computes each joint frame's joint-bin plane (one byte per
+ * pixel, in its workspace).  A zero-initialised struct is a uniform one-channel
  * frame. */
 typedef struct {
   int h, w, nbins, layout;
@@ -420,7 +433,7 @@ int ihist_batch_get_tune(ihist_batch_t batch, ihist_tune_t *out);
  * Nothing is allocated. */
 int ihist_batch_set_io(ihist_batch_t batch, const ihist_frame_t *frames, int n, void *stream);
 
-/* Compute every bound frame of the batch in one launch on `stream`.  Bindings
+/* Compute every bound frame of the batch on `stream`.  Bindings
  * and launches may be on different streams: a live launch of the two-launch
  * path runs after its binding's copies, and a later binding's copies after it. */
 int ihist_batch_compute(ihist_batch_t batch, void *stream);

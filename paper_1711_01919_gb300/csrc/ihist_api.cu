@@ -823,7 +823,7 @@ static void launch_sorted_group(const uint32_t *hist, int H, int W, int B, int b
 }
 
 // Bins of one pass where the caller leaves it open: 16 (2^20 rectangles x 128
-// bins on 8192 x 8192 4.36 ms, 8 bins 4.76; 204,682 x 37 on 2432 x 2545 250
+// bins on 8192 x 8192 4.36-4.98 ms, 8 bins 4.76-5.66; 204,682 x 37 on 2432 x 2545 250
 // and 278 us), or 8 for a histogram of no more (146,420 x 8 on 512 x 512 77 us,
 // 16 bins 86).
 static int sorted_group(int nbins, int bins_per_pass) {

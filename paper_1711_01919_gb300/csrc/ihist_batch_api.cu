@@ -1,6 +1,7 @@
 // ihist_batch_api.cu -- host side of libihist.so for batches: one persistent
-// launch over many frames of uneven size (slot planning, rebinding, uploads,
-// launches and queries).  Declared in include/ihist.h.
+// launch, or the two-launch path's, over many frames of uneven size (slot
+// planning, rebinding, uploads, launches and queries).  Declared in
+// include/ihist.h.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
@@ -273,7 +274,7 @@ static bool encode_frame_map(const uint8_t *in, size_t pitch, int h, int w, int 
 //    own here, so from some number of pixels on that kernel is faster (two
 //    launches against one, us): 24 frames of 1920x1080 x 4 214 / 205, 128 of
 //    640x480 x 4 171 / 157, 64 of 1920x1080 x 2 1.11x, x 4 565 / 457, x 8 885 /
-//    800, x 6 (two bins of the second group to write) 1.04x, x 12 1.06x, x 16 1.03x, x 24 1.01x, but 16 of them x 4 0.93x, 24 x 8
+//    800, x 6 1.04x, x 12 1.06x, x 16 1.03x, x 24 1.01x, but 16 of them x 4 0.93x, 24 x 8
 //    0.99x.  It takes about twice as many where frames are wider than 16 chunks,
 //    which fill that kernel's CTAs less evenly (3840x2160 x 4: 6, 12 and 32
 //    frames 0.98x, 1.05x, 1.24x, x 8: 12 and 32 0.98x, 1.09x).  Quad-major:

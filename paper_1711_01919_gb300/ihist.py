@@ -629,8 +629,8 @@ def out_shape(h: int, w: int, nbins: int, layout: int):
 
 
 class Batch:
-    """Many frames (CUDA uint8 [h][w] tensors, any mix of shapes) in one
-    persistent launch; outputs are int32 tensors holding uint32 counts."""
+    """Many frames (CUDA uint8 [h][w] tensors, any mix of shapes) per launch;
+    outputs are int32 tensors holding uint32 counts."""
 
     def __init__(self, frames, nbins, layouts=None, outs=None, tune=None, tables=None, joint=None):
         """tables: None, or one entry per frame, None (uniform bins) or a
